@@ -41,34 +41,30 @@ if ROOT not in sys.path:
 
 N_CAMERAS = 20
 L2_FLUSH_BYTES = 256 << 20
-# FP32 operations per evaluated blob in the compositor: 3 sub, 1 mul + 2 fma (squared
-# distance), 1 fma (scaled exponent plus log2 amplitude), 1 add (density), 3 fma (colour);
-# the exp2 runs on the MUFU pipe alongside.  The compositor evaluates two samples per
-# lane with paired (f32x2) instructions, so this is 5.5 instructions per evaluation.  It
-# skips blobs beyond 7 s of a chunk's points by definition; the library counts the
+# FP32 operations per evaluated blob in the compositor: 2 fma (the exponent along the ray),
+# 1 add (density), 3 fma (colour); the exp2 runs on the MUFU pipe alongside.  The
+# compositor evaluates samples in pairs (f32x2), so this is 3 instructions per evaluation.
+# It skips blobs beyond 7 s of a chunk's points by definition; the library counts the
 # evaluations it does make when its work counters are on ("composite_blob_evals"), which
 # the bench does in a separate untimed pass.
-COMPOSITE_FP32_PER_BLOB = 11
+COMPOSITE_FP32_PER_BLOB = 6
 KERNELS_PER_TIMER = {"build_vdb": 5}   # the builder's timer spans five kernels
 # L2 hit rate and warp execution efficiency (active lanes per warp instruction) per kernel
 # from the ncu --set full captures (object frame, camera 0; unbounded: its first 200 image
 # rows); dropped like the traffic when a kernel changes.
 PROFILED_COUNTERS = {
     "object": {"hdda_walk": {"l2_hit_pct": 53.8, "active_lanes_of_32": 26.06},
-               "hdda_emit": {"l2_hit_pct": 10.7, "active_lanes_of_32": 27.16},
-               "composite": {"l2_hit_pct": 26.4, "active_lanes_of_32": 30.03}},
+               "hdda_emit": {"l2_hit_pct": 10.7, "active_lanes_of_32": 27.16}},
     "unbounded": {"hdda_walk": {"l2_hit_pct": 56.7, "active_lanes_of_32": 26.01},
-                  "hdda_emit": {"l2_hit_pct": 10.0, "active_lanes_of_32": 30.15},
-                  "composite": {"l2_hit_pct": 16.6, "active_lanes_of_32": 30.46}},
+                  "hdda_emit": {"l2_hit_pct": 10.0, "active_lanes_of_32": 30.15}},
 }
 # DRAM bytes (read + write) per launch from ncu of a workload's step on camera 0 (the
 # capture commands are kept with the profile summaries), for the roofline's "traffic"; an
 # entry must be dropped whenever its kernel changes, and a workload without a capture
 # reports none.
 PROFILED_TRAFFIC = {
-    "object": {"composite": 233_599_744, "hdda_emit": 266_574_592, "hdda_walk": 16_295_424},
-    "unbounded": {"composite": 1_502_165_760, "hdda_emit": 2_182_214_144,
-                  "hdda_walk": 27_365_888},
+    "object": {"hdda_emit": 266_574_592, "hdda_walk": 16_295_424},
+    "unbounded": {"hdda_emit": 2_182_214_144, "hdda_walk": 27_365_888},
 }
 
 

@@ -448,7 +448,7 @@ void hdda_batch_free(hdda_batch* batch);
  *   t0, t1          device float samples
  *   field           device float [n_gauss][8] = mu_x, mu_y, mu_z, s, a, r, g, b,
  *                   with s > 0 and a >= 0.  A blob is skipped for a group of
- *                   64 consecutive samples when it lies farther than 7 s from
+ *                   up to 32 samples of one ray when it lies farther than 7 s from
  *                   every one of them (its weight there is below a * e^-24.5);
  *                   the distance tests keep a small margin for rounding, so
  *                   no blob within 7 s of a sample is skipped
@@ -518,9 +518,8 @@ int hdda_traverse_composite(const float* rays_o, const float* rays_d, int64_t n_
  *                          by two CUDA events recorded on its stream (one
  *                          event pair per launch)
  *   HDDA_PROFILE_COUNTERS  the compositors count blob evaluations (sample x
- *                          kept blob), one atomic add per warp task; this
- *                          is extra device work, so time with the timers
- *                          alone
+ *                          kept blob), one atomic add per ray; this is
+ *                          extra device work, so time with the timers alone
  * hdda_profiler_enable(flags) sets both switches (0 turns everything off).
  * hdda_profiler_read synchronises on the recorded events, writes up to `cap`
  * per-kernel aggregates (HOST array) and clears them; *n_out (HOST)

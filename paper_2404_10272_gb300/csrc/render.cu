@@ -5,21 +5,21 @@
 //
 // Pass 1 is the samplers' walk (walk_kernel, walk.cuh): each ray's merged
 // occupied runs of lattice indices [k_begin, k_end), the first kMaxRuns of
-// them, and its number of runs.  Pass 2 (render_kernel) gives each warp 8
-// consecutive rays (measured faster than 4 or 16).  Every
-// lattice index k of a run is the sample (t_k, t_{k+1}) with midpoint tm_k,
-// read from the lattice table all rays share, so a warp numbers its rays'
-// samples locally (a warp scan of the run lengths), and each sample of a
-// 64-sample chunk (two per lane, field.cuh) finds its ray (compares against
-// the slots' first positions, kept in registers) and its run (binary search
-// over that ray's runs in shared memory).  The task's rays are staged in
-// shared memory.  No global scan, no sample arrays, no host read-back.
+// them, and its number of runs.  Pass 2 (render_kernel) gives each warp R
+// consecutive rays (field_task_rays), four of them in work at a time, one
+// per group of eight lanes, 32 samples per step (field.cuh).  Every lattice
+// index k of a run is the sample (t_k, t_{k+1}), read from the lattice table
+// all rays share.  The task's runs are staged in shared memory with their
+// first sample positions in the ray, so that a lane finds the run of its
+// four consecutive samples by a binary search; usually they lie in one run
+// and are five consecutive lattice entries.  No global scan, no sample
+// arrays, no host read-back.
 //
 // A ray with more than kMaxRuns runs is finished in rounds: after the runs
 // it has are composited, it walks again from the end of the last one
-// (walk_from) and the next kMaxRuns runs are composited with its
-// transmittance and colour carried over, so samples are still accumulated
-// front to back.
+// (walk_from) and the next kMaxRuns runs are composited with its optical
+// depth and colour carried over, so samples are still accumulated front to
+// back.
 //
 // The same kernel with kStore also writes what the samplers' emit writes:
 // the CSR offsets (each task's 32-ray tile prefix from the tile scan plus a
@@ -34,8 +34,8 @@ namespace hdda {
 namespace {
 
 constexpr int kRenderWarps = 4;
-constexpr int kRenderRays = 8;  // rays per warp task
 constexpr uint32_t kNoRun = 0x7fffffffu;
+constexpr int kRunStride = kMaxRuns + 1;  // per ray: odd, so the groups' searches hit other banks
 
 // Blob evaluations (sample x kept blob), counted only while profiling.
 __device__ unsigned long long g_render_evals;
@@ -52,81 +52,75 @@ struct StoreArgs {
   unsigned* status;            // kDevCapacity when the samples do not fit
 };
 
-// Position p of a round (numbered over the warp's rays) -> its lattice index:
-// the run j of slot `own` that starts at or before p.  Runs hold {first k,
-// first position}; unused slots have position kNoRun.
-__device__ __forceinline__ int run_k(const uint2* sr, int own, int p, int& j) {
-  j = 0;
-#pragma unroll
-  for (int s = kMaxRuns / 2; s > 0; s >>= 1)
-    if (sr[(j + s) * kRenderRays + own].y <= (uint32_t)p) j += s;
-  const uint2 e = sr[j * kRenderRays + own];
-  return (int)e.x + (p - (int)e.y);
+// Turns a ray's `nr` runs [k_begin, k_end) into {k_begin - first position,
+// first position}, positions counted within the ray's round (unused slots
+// start at kNoRun, as does the one after the last), and returns the number of
+// samples.
+__device__ __forceinline__ int number_runs(uint2* sr, int nr) {
+  int pos = 0;
+  for (int j = 0; j < kRunStride; ++j) {
+    const uint2 v = sr[j];
+    if (j < nr) {
+      sr[j] = make_uint2(v.x - (uint32_t)pos, (uint32_t)pos);
+      pos += (int)(v.y - v.x);
+    } else {
+      sr[j] = make_uint2(0u, kNoRun);
+    }
+  }
+  return pos;
 }
 
-template <int kMode, bool kStore>
+template <int kMode, bool kStore, bool kMany>
 __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
-    const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, GridDev g,
+    const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R, GridDev g,
     LatticeDev lat, const uint8_t* __restrict__ nruns, const uint2* __restrict__ runs,
     const float* __restrict__ field, int G, float* __restrict__ rgba, bool count_evals,
     StoreArgs out) {
-  extern __shared__ __align__(16) unsigned char smem[];  // field_smem_bytes(G, kRenderWarps)
-  __shared__ float s_T[kRenderWarps][kRenderRays];
-  __shared__ float4 s_C[kRenderWarps][kRenderRays];
-  __shared__ uint16_t s_cand[kRenderWarps][kMaxGauss];  // the task's candidate blobs
-  __shared__ float4 s_ray[kRenderWarps][kRenderRays][2];  // {o, d.x}, {d.y, d.z, 1/|d|^2, -}
-  __shared__ int64_t s_gbase[kRenderWarps][kRenderRays];  // storing form: output of position 0
-  // run j of ray slot i at [j * kRenderRays + i]: {first k, first position}
-  __shared__ uint2 s_run[kRenderWarps][kMaxRuns * kRenderRays];
-  const FieldSmem fs = stage_blobs(smem, field, G);
+  // field_layout(G, kRenderWarps, R), then [kRenderWarps][R][kRunStride] runs
+  extern __shared__ __align__(16) unsigned char smem[];
+  const FieldLayout L = field_layout(G, kRenderWarps, R);
+  stage_blobs(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t task = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (task * kRenderRays >= n) return;  // uniform per warp; no block barrier follows
-  float* T_s = s_T[wib];
-  float4* C_s = s_C[wib];
-  float4 (*rs)[2] = s_ray[wib];
-  int64_t* gb = s_gbase[wib];
-  uint2* sr = s_run[wib];
-  unsigned long long evals = 0;  // this warp's blob evaluations
-  const LatHdr h = lat_hdr(lat);
-  const int64_t r = task * kRenderRays + lane;
-  const bool has_ray = lane < kRenderRays && r < n;
-  bool ok = false;
-  if (lane < kRenderRays) {
-    // the ray stays in shared memory only; a ray that needs another round of
-    // runs rebuilds its walk state from there
-    float o[3] = {0.f, 0.f, 0.f}, d[3] = {0.f, 0.f, 0.f};
-    if (has_ray) {
-      ok = true;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        o[c] = __ldg(ro + 3 * r + c);
-        d[c] = __ldg(rd + 3 * r + c);
-        ok &= isfinite(o[c]) && isfinite(d[c]);
-      }
-    }
-    T_s[lane] = 1.f;
-    C_s[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
-    rs[lane][0] = make_float4(o[0], o[1], o[2], d[0]);
-    rs[lane][1] = make_float4(d[1], d[2], dd > 1e-30f ? 1.f / dd : 0.f, 0.f);
+  const int grp = lane / kGroupLanes, gl = lane & (kGroupLanes - 1);
+  const int64_t task = (int64_t)blockIdx.x * kRenderWarps + wib, first = task * R;
+  if (first >= n) return;  // uniform per warp; no block barrier follows
+  FieldWarp<kMany> fw;
+  fw.init(smem, L);
+  uint2* sr = reinterpret_cast<uint2*>(smem + L.bytes) + wib * R * kRunStride;
+
+  // lane i < R holds ray i's number of runs, samples of this round and resume index
+  const int64_t r = first + lane;
+  const bool has_ray = lane < R && r < n;
+  const int nr_all = has_ray ? (int)__ldg(nruns + r) : 0;  // saturated at 255; 0 when not finite
+  const int nr = min(nr_all, kMaxRuns);
+  for (int u0 = 0; u0 < R * kMaxRuns; u0 += 32) {  // R is a multiple of 4: at least two slots
+    const int u = u0 + lane, i = u & (R - 1), j = u / R;
+    if (j < __shfl_sync(kFull, nr, i)) sr[i * kRunStride + j] = __ldg(runs + (int64_t)j * n + first + i);
   }
   __syncwarp();
-  uint16_t* cand = s_cand[wib];
-  const int ncand =
-      task_candidates(fs, G, rs, (int)min((int64_t)kRenderRays, n - task * kRenderRays), cand);
-  const int nr_all = ok ? (int)nruns[r] : 0;  // saturated at 255
-  int nr = min(nr_all, kMaxRuns);
-  for (int j = 0; j < nr; ++j) sr[j * kRenderRays + lane] = __ldg(runs + (int64_t)j * n + r);
-  int k_next = lat.K;  // where the ray's walk resumes
-  if (nr_all > kMaxRuns) k_next = (int)sr[(kMaxRuns - 1) * kRenderRays + lane].y;
-  // storing form: lane i < kRenderRays holds ray i's CSR offset, then, per
-  // round, the output position of the round's position 0 of that ray
-  int64_t gofs = 0;
+  int my_w = 0, my_next = lat.K;
+  if (nr > 0) {
+    const uint32_t ka = sr[lane * kRunStride].x, kb = sr[lane * kRunStride + nr - 1].y;
+    if (nr_all > kMaxRuns) my_next = (int)kb;
+    const float tb = 0.5f * (__ldg(lat.t + ka) + __ldg(lat.t + kb));
+    float o[3], d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      o[c] = __ldg(ro + 3 * r + c);
+      d[c] = __ldg(rd + 3 * r + c);
+    }
+    make_ray_rec(fw.rays(L) + lane, o, d, tb);
+    my_w = number_runs(sr + lane * kRunStride, nr);
+  } else if (has_ray) {
+    reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  unsigned pending = __ballot_sync(kFull, nr > 0);  // rays not yet taken by a group
+  // storing form: the ray's CSR offset
+  int64_t my_gofs = 0;
   if constexpr (kStore) {
-    constexpr int kTasksPerTile = 32 / kRenderRays;
-    const int64_t tile = task / kTasksPerTile;
+    const int per_tile = 32 / R;  // R divides 32
+    const int64_t tile = task / per_tile;
     const int64_t tr = tile * 32 + lane;
     const int64_t c = tr < n ? (int64_t)__ldg(out.counts + tr) : 0;
     int64_t inc = c;
@@ -136,126 +130,173 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
       if (lane >= o) inc += y;
     }
     const int64_t ex = __ldg(out.tile_prefix + tile) + inc - c;
-    const int first = (int)(task % kTasksPerTile) * kRenderRays;
-    gofs = __shfl_sync(kFull, ex, first + (lane & (kRenderRays - 1)));
-    const int64_t mine = __shfl_sync(kFull, c, first + (lane & (kRenderRays - 1)));
+    const int slot = (int)(task % per_tile) * R + (lane & (R - 1));
+    my_gofs = __shfl_sync(kFull, ex, slot);
+    const int64_t mine = __shfl_sync(kFull, c, slot);
     // capacity 0 counts only: offsets unclamped, no samples, no status
     const bool clamp = out.capacity > 0;
     if (has_ray) {
-      out.offsets[r] = clamp ? min(gofs, out.capacity) : gofs;
-      if (r == n - 1) out.offsets[n] = clamp ? min(gofs + mine, out.capacity) : gofs + mine;
+      out.offsets[r] = clamp ? min(my_gofs, out.capacity) : my_gofs;
+      if (r == n - 1)
+        out.offsets[n] = clamp ? min(my_gofs + mine, out.capacity) : my_gofs + mine;
     }
-    if (__any_sync(kFull, clamp && has_ray && gofs + mine > out.capacity) && lane == 0)
+    if (__any_sync(kFull, clamp && has_ray && my_gofs + mine > out.capacity) && lane == 0)
       atomicOr(out.status, kDevCapacity);
   }
+  __syncwarp();
+
+  // the group's ray: its index in the task (-1: none), samples of this round,
+  // the lane's position, resume index, records
+  int ray = -1, W = 0, q = 0, k_next = 0;
+  float tb = 0.f;
+  int64_t gofs = 0;
+  unsigned evals = 0;  // of the ray in work
+  RayAcc acc;
+  acc_clear(acc);
+  rgba += 4 * first;
   for (;;) {
-    // this round's runs: lengths, the warp's numbering, then first positions
-    int cnt = 0;
-    for (int j = 0; j < nr; ++j) {
-      const uint2 v = sr[j * kRenderRays + lane];
-      cnt += (int)(v.y - v.x);
+    unsigned idle = __ballot_sync(kFull, ray < 0) & kLeaders;  // one bit per group
+    if (idle) {  // uniform
+      if (!pending && idle == kLeaders) break;
+      while (idle && pending) {
+        const int gi = (__ffs(idle) - 1) / kGroupLanes, i = __ffs(pending) - 1;
+        idle &= idle - 1;
+        pending &= pending - 1;
+        const int w = __shfl_sync(kFull, my_w, i), kn = __shfl_sync(kFull, my_next, i);
+        int64_t go = 0;
+        if constexpr (kStore) go = __shfl_sync(kFull, my_gofs, i);
+        if (grp == gi) {
+          ray = i;
+          W = w;
+          k_next = kn;
+          q = kPerLane * gl;
+          tb = fw.rays(L)[i].base.w;
+          gofs = go;
+        }
+        fw.setup(L, G, gi, i);
+      }
+      fw.ready();
     }
-    int inc = cnt;
+    // this chunk's samples
+    float2 a[kPairs], b[kPairs];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += y;
-    }
-    const int pos = inc - cnt;
-    const int W = __shfl_sync(kFull, inc, 31);
-    // every lane keeps the first positions of slots 1 .. kRenderRays - 1
-    int q[kRenderRays];
+    for (int h = 0; h < kPairs; ++h) a[h] = b[h] = splat(tb);
+    if (ray >= 0 && q < W) {
+      const uint2* mr = sr + ray * kRunStride;
+      int j = 0;  // the last run that starts at or before q
 #pragma unroll
-    for (int i = 1; i < kRenderRays; ++i) q[i] = __shfl_sync(kFull, pos, i);
-    if (lane < kRenderRays) {
-      if constexpr (kStore) gb[lane] = gofs - pos;
-      int qq = pos;
-      for (int j = 0; j < kMaxRuns; ++j) {
-        uint2& e = sr[j * kRenderRays + lane];
-        if (j < nr) {
-          const int len = (int)(e.y - e.x);
-          e.y = (uint32_t)qq;
-          qq += len;
-        } else {
-          e = make_uint2(0u, kNoRun);
+      for (int s = kMaxRuns / 2; s > 0; s >>= 1)
+        if (mr[j + s].y <= (uint32_t)q) j += s;
+      uint32_t kq = mr[j].x;
+      uint32_t nxt = mr[j + 1].y;
+      if ((uint32_t)(q + kPerLane) <= nxt && q + kPerLane <= W) {
+        const float* t = lat.t + (int)(kq + (uint32_t)q);
+        float x = __ldg(t);
+#pragma unroll
+        for (int h = 0; h < kPairs; ++h) {
+          const float y = __ldg(t + 2 * h + 1), z = __ldg(t + 2 * h + 2);
+          a[h] = make_float2(x, y);
+          b[h] = make_float2(y, z);
+          x = z;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < kPerLane; ++i) {
+          if (q + i >= W) continue;
+          if ((uint32_t)(q + i) >= nxt) {  // a run holds at least one sample
+            kq = mr[++j].x;
+            nxt = mr[j + 1].y;
+          }
+          const float* t = lat.t + (int)(kq + (uint32_t)(q + i));
+          (i & 1 ? a[i / 2].y : a[i / 2].x) = __ldg(t);
+          (i & 1 ? b[i / 2].y : b[i / 2].x) = __ldg(t + 1);
         }
       }
-    }
-    __syncwarp();
-    for (int base = 0; base < W; base += kChunk) {
-      Elem e[2];
-      int k0 = 0, j0 = 0;
+      if constexpr (kStore) {
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const int p = base + 2 * lane + hh;
-        int own = 0;  // the last slot whose first position is <= p
-#pragma unroll
-        for (int i = 1; i < kRenderRays; ++i) own += p >= q[i];
-        e[hh].own = own;
-        e[hh].a0 = e[hh].a1 = e[hh].px = e[hh].py = e[hh].pz = 0.f;
-        if (p < W) {
-          int k;
-          if (hh == 1 && own == e[0].own &&
-              (j0 + 1 >= kMaxRuns || (uint32_t)p < sr[(j0 + 1) * kRenderRays + own].y)) {
-            // the next lattice index of e0's run: its start is e0's end
-            k = k0 + 1;
-            e[1].a0 = e[0].a1;
-          } else {
-            int j;
-            k = run_k(sr, own, p, j);
-            e[hh].a0 = __ldg(lat.t + k);
-            k0 = k;
-            j0 = j;
-          }
-          e[hh].a1 = __ldg(lat.t + k + 1);
-          // the midpoint as the lattice defines it: fl(fl(t_k + t_k+1) * 0.5)
-          const float tm = __fmul_rn(__fadd_rn(e[hh].a0, e[hh].a1), 0.5f);
-          const float4 A = rs[own][0], B = rs[own][1];
-          e[hh].px = fmaf(tm, A.w, A.x);
-          e[hh].py = fmaf(tm, B.x, A.y);
-          e[hh].pz = fmaf(tm, B.y, A.z);
-          if constexpr (kStore) {
-            const int64_t qo = gb[own] + p;
-            if (qo < out.capacity) {
-              out.ray_idx[qo] = (int32_t)(task * kRenderRays + own);
-              out.t0[qo] = e[hh].a0;
-              out.t1[qo] = e[hh].a1;
-            }
+        for (int i = 0; i < kPerLane; ++i) {
+          const int64_t qo = gofs + q + i;
+          if (q + i < W && qo < out.capacity) {
+            out.ray_idx[qo] = (int32_t)(first + ray);
+            out.t0[qo] = i & 1 ? a[i / 2].y : a[i / 2].x;
+            out.t1[qo] = i & 1 ? b[i / 2].y : b[i / 2].x;
           }
         }
       }
-      evals += composite_chunk2(fs, cand, ncand, min(kChunk, W - base), e[0], e[1], rs, T_s, C_s);
     }
-    if constexpr (kStore) gofs += cnt;  // this round's samples of the lane's ray are written
-    const bool more = k_next < lat.K;
-    if (!__any_sync(kFull, more)) break;
-    nr = 0;
-    if (more) {
-      Ray ray;
-      const float4 A = rs[lane][0], B = rs[lane][1];
-      const float o[3] = {A.x, A.y, A.z}, d[3] = {A.w, B.x, B.y};
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {  // as load_ray (walk.cuh) sets them up
-        ray.o[c] = o[c];
-        ray.d[c] = d[c];
-        ray.neg[c] = d[c] < 0.f;
-        ray.inv[c] = d[c] != 0.f ? 1.0f / d[c] : INFINITY;
+    float2 t[kPairs], dt[kPairs];
+    float lo, hi;
+    chunk_params(a, b, tb, q, W, t, dt, lo, hi);
+    int kept;
+    const int len = fw.cull(L, G, lo, hi, kept);
+    BlobSums sums;
+    sums_clear(sums);
+    sum_blobs(smem, fw.recs + L.list, len, t, sums);
+    if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
+    if (count_evals && ray >= 0 && gl == 0)
+      evals += (unsigned)kept * (unsigned) min(kChunk, W - q);
+    shade_chunk(sums, dt, acc);
+    q += kChunk;
+    const bool round_over = ray >= 0 && q - kPerLane * gl >= W;
+    bool done = round_over && k_next >= lat.K;
+    if (__any_sync(kFull, round_over && !done)) {  // another round of runs for these groups
+      int nr2 = 0;
+      if (round_over && !done) {
+        gofs += W;
+        if (gl == 0) {
+          uint2* mr = sr + ray * kRunStride;
+          Ray ry;
+          load_ray(ro, rd, first + ray, ry);
+          const LatHdr h = lat_hdr(lat);
+          k_next = walk_from<kMode, false>(g, global_tabs(g), lat, h, ry, k_next, mr, 1, nr2);
+          W = number_runs(mr, nr2);
+        }
       }
-      k_next = walk_from<kMode, false>(g, global_tabs(g), lat, h, ray, k_next, sr + lane,
-                                       kRenderRays, nr);
+      const int w = __shfl_sync(kFull, W, lane & ~(kGroupLanes - 1));
+      const int kn = __shfl_sync(kFull, k_next, lane & ~(kGroupLanes - 1));
+      if (round_over && !done) {
+        W = w;
+        k_next = kn;
+        q = kPerLane * gl;
+        done = W == 0;
+      }
     }
-    __syncwarp();
+    if (__any_sync(kFull, done)) {
+      finish_rays(acc, done, rgba + 4 * ray);
+      if (done) {
+        ray = -1;
+        W = 0;
+        fw.release();
+        acc_clear(acc);
+        if (count_evals && gl == 0) atomicAdd(&g_render_evals, (unsigned long long)evals);
+        evals = 0;
+      }
+    }
+    __syncwarp();  // the group's lists, records and runs may be overwritten
   }
-  if (has_ray) {
-    const float4 acc = C_s[lane];
-    reinterpret_cast<float4*>(rgba)[r] = make_float4(acc.x, acc.y, acc.z, 1.f - T_s[lane]);
-  }
-  if (count_evals && lane == 0) atomicAdd(&g_render_evals, evals);
 }
 
 const char* render_name(int mode) {
   return mode == kModeDense ? "dense_render" : mode == kModeVdb ? "hdda_render_plain"
                                                                  : "hdda_render";
+}
+
+template <int kMode, bool kStore>
+int launch_field(const WalkArgs& w, const uint8_t* nr, const uint2* runs, const float* field,
+                 int G, float* rgba, const StoreArgs& out, cudaStream_t s) {
+  const int R = field_task_rays(w.n);
+  const int64_t warps = (w.n + R - 1) / R;
+  const unsigned nb = (unsigned)((warps + kRenderWarps - 1) / kRenderWarps);
+  const size_t smem = field_layout(G, kRenderWarps, R).bytes +
+                      (size_t)kRenderWarps * R * kRunStride * sizeof(uint2);
+  const auto kern =
+      G <= kAllBlobs ? render_kernel<kMode, kStore, false> : render_kernel<kMode, kStore, true>;
+  if (smem > 48 * 1024)
+    HDDA_CUDA_TRY(
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kern<<<nb, kRenderWarps * 32, smem, s>>>(w.ro, w.rd, w.n, R, w.g, w.lat, nr, runs, field, G, rgba,
+                                           counters_on(), out);
+  return HDDA_OK;
 }
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -299,24 +340,13 @@ int launch_render(const float* ro, const float* rd, int64_t n, const hdda_grid* 
   }
   {
     KernelTimer kt(render_name(mode), s);
-    const int64_t warps = (n + kRenderRays - 1) / kRenderRays;
-    const unsigned nb = (unsigned)((warps + kRenderWarps - 1) / kRenderWarps);
-    const bool ev = counters_on();
-    const size_t fsm = field_smem_bytes(G, kRenderWarps);
-    switch (mode) {
-      case kModeDense:
-        render_kernel<kModeDense, false><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, StoreArgs{});
-        break;
-      case kModeVdb:
-        render_kernel<kModeVdb, false><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, StoreArgs{});
-        break;
-      default:
-        render_kernel<kModeVdbMap, false><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, StoreArgs{});
-        break;
-    }
+    const StoreArgs none{};
+    const int st = mode == kModeDense
+                       ? launch_field<kModeDense, false>(w, nr, runs, field, G, rgba, none, s)
+                   : mode == kModeVdb
+                       ? launch_field<kModeVdb, false>(w, nr, runs, field, G, rgba, none, s)
+                       : launch_field<kModeVdbMap, false>(w, nr, runs, field, G, rgba, none, s);
+    if (st != HDDA_OK) return st;
   }
   HDDA_CUDA_TRY(cudaGetLastError());
   return HDDA_OK;
@@ -381,25 +411,13 @@ int launch_sample_composite(const float* ro, const float* rd, int64_t n, const h
   HDDA_CUDA_TRY(cudaGetLastError());
   {
     KernelTimer kt(sample_composite_name(mode), s);
-    const int64_t warps = (n + kRenderRays - 1) / kRenderRays;
-    const unsigned nb = (unsigned)((warps + kRenderWarps - 1) / kRenderWarps);
-    const bool ev = counters_on();
-    const size_t fsm = field_smem_bytes(G, kRenderWarps);
     const StoreArgs out{tile_prefix, counts, offsets, ray_idx, t0, t1, capacity, status};
-    switch (mode) {
-      case kModeDense:
-        render_kernel<kModeDense, true><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, out);
-        break;
-      case kModeVdb:
-        render_kernel<kModeVdb, true><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, out);
-        break;
-      default:
-        render_kernel<kModeVdbMap, true><<<nb, kRenderWarps * 32, fsm, s>>>(
-            ro, rd, n, w.g, lat, nr, runs, field, G, rgba, ev, out);
-        break;
-    }
+    const int st = mode == kModeDense
+                       ? launch_field<kModeDense, true>(w, nr, runs, field, G, rgba, out, s)
+                   : mode == kModeVdb
+                       ? launch_field<kModeVdb, true>(w, nr, runs, field, G, rgba, out, s)
+                       : launch_field<kModeVdbMap, true>(w, nr, runs, field, G, rgba, out, s);
+    if (st != HDDA_OK) return st;
   }
   HDDA_CUDA_TRY(cudaGetLastError());
   return HDDA_OK;

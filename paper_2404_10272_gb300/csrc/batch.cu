@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kBlock) batch_walk_kernel(
         Ray ray;
         int nr = 0;
         if (load_ray(ro, rd, lr, ray))
-          c = walk<kMode, false, false, kSkip, kCheck>(g, global_tabs(g), lat, h, ray, runs + gr,
+          c = walk<kMode, false, false, kSkip, kCheck>(g, global_tabs(g, lat), lat, h, ray, runs + gr,
                                                        slots, nr, 0, 0, 0, nullptr, nullptr,
                                                        nullptr, status);
         counts[gr] = (int32_t)c;
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
       load_ray(jb.ro, jb.rd, lr, ray);
       const LatHdr h = lat_hdr(lat);
       int unused = 0;
-      walk<kMode, true, false>(s_grid[warp], global_tabs(s_grid[warp]), lat, h, ray, nullptr, 0,
+      walk<kMode, true, false>(s_grid[warp], global_tabs(s_grid[warp], lat), lat, h, ray, nullptr, 0,
                                unused, (int32_t)lr, off, capacity, jb.ray_idx, jb.t0, jb.t1,
                                status);
     }

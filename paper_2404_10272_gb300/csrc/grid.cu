@@ -38,7 +38,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-__global__ void thresholds_kernel(GridDev g, float* __restrict__ thr) {
+__global__ void thresholds_kernel(GridDev g, float* __restrict__ thr, float* __restrict__ mthr) {
   const int64_t R1 = g.R + 1;
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)g.L * 3 * R1) return;
@@ -65,6 +65,17 @@ __global__ void thresholds_kernel(GridDev g, float* __restrict__ thr) {
     X = key_float(kh);
   }
   thr[idx] = X;
+  // the mirrored bounds (hdda_internal.cuh)
+  float* m = mthr + (int64_t)lc * mthr_stride(g.R) + g.R;
+  if (a < g.R) {
+    const uint32_t u = __float_as_uint(X);
+    const float below = (u & 0x7fffffffu) == 0u ? __uint_as_float(0x80000001u)
+                                                 : __uint_as_float((u & 0x80000000u) ? u + 1u : u - 1u);
+    m[-a - 1] = -below;
+  }
+  if (a > 0) m[a - 1] = X;
+  if (a == g.R)
+    for (int j = 0; j < kNodeVox; ++j) m[g.R + j] = X;
 }
 
 __global__ void pack_dense_kernel(const uint8_t* __restrict__ dense, int L, int R, int W,
@@ -567,6 +578,7 @@ size_t layout(hdda_grid* g, char* base) {
   const bool vdb = g->kind == HDDA_GRID_VDB;
   size_t off = 0;
   carve(base, off, g->thr, g->thr_count(), true);
+  carve(base, off, g->mthr, (int64_t)g->L * 3 * mthr_stride(g->R), true);
   carve(base, off, g->bits, (int64_t)g->L * g->W, !vdb);
   const int64_t nw = g->nodes_total() * kNodeWords;
   carve(base, off, g->child, nw, vdb);
@@ -652,7 +664,7 @@ int create(int kind, const uint8_t* dense, int levels, int res, const hdda_aabb*
   layout(g, static_cast<char*>(g->base));
   e = cudaEventCreateWithFlags(&g->built, cudaEventDisableTiming);
   if (e != cudaSuccess) { hdda_grid_free(g); return cuda_error(e, "cudaEventCreate"); }
-  thresholds_kernel<<<blocks_for(g->thr_count(), 128), 128, 0, s>>>(g->view(), g->thr);
+  thresholds_kernel<<<blocks_for(g->thr_count(), 128), 128, 0, s>>>(g->view(), g->thr, g->mthr);
   e = cudaGetLastError();
   if (e != cudaSuccess) { hdda_grid_free(g); return cuda_error(e, "thresholds_kernel"); }
   st = launch_build(g, dense, s);

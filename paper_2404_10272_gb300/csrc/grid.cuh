@@ -15,6 +15,7 @@ struct hdda_grid {
   size_t base_bytes = 0;
 
   float* thr = nullptr;          // [L][3][R+1]
+  float* mthr = nullptr;         // [L][3][mthr_stride(R)]
   uint32_t* bits = nullptr;      // dense [L][W]
   uint32_t* child = nullptr;     // vdb [L*N^3][128]
   uint32_t* tile = nullptr;      // vdb [L*N^3][128]
@@ -55,7 +56,7 @@ struct hdda_grid {
         g.lv[l].s[c] = scale[l][c];
       }
     }
-    g.thr = thr; g.bits = bits; g.child = child; g.tile = tile;
+    g.thr = thr; g.mthr = mthr; g.bits = bits; g.child = child; g.tile = tile;
     g.prefix = prefix; g.nstate = nstate; g.leaves = leaves;
     g.nsuper = nsuper; g.lsub = lsub; g.rmap = rmap;
     g.check = hdda::region_checks_on() ? 1 : 0;

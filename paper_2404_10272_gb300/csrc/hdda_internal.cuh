@@ -69,6 +69,7 @@ struct GridDev {
   int W;                     // dense bit words per level
   LevelDev lv[kMaxLevels];
   const float* thr;          // [L][3][R+1] exact index thresholds
+  const float* mthr;         // [L][3][mthr_stride(R)] the same as mirrored upper bounds
   const uint32_t* bits;      // dense: [L][W]
   const uint32_t* child;     // vdb: [L*N^3][128]
   const uint32_t* tile;      // vdb: [L*N^3][128]
@@ -102,6 +103,16 @@ __host__ __device__ constexpr size_t lattice_block_bytes(int max_k) {
   return (sizeof(float) * (2 * (size_t)max_k + 1) + sizeof(int) * (kKidxMax + 2) + 32 + 255) &
          ~(size_t)255;
 }
+
+// The thresholds as a walk reads them (mthr): the upper bound, exclusive, of
+// the aligned cube of szm + 1 voxels (szm + 1 a power of two up to 128) that
+// holds voxel i, in the coordinate of a ray that moves up (mirror mask m = 0)
+// or, negated, down (m = all ones) this axis, is entry R + ((i ^ m) | szm):
+//   m = 0   index a1 - 1, a1 the cube's end: X[min(a1, R)]
+//   m = ~0  index -a0 - 1, a0 its start: -(the value below X[a0]), because
+//           x < X[a0] is -x >= that
+// so both directions take one load and no clamp (128 entries of padding).
+__host__ __device__ constexpr int mthr_stride(int R) { return 2 * R + kNodeVox; }
 
 __device__ __forceinline__ int voxel_index(float x, float lo, float s, int R) {
   float u = __fmul_rn(__fsub_rn(x, lo), s);

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
           Ray ry;
           load_ray(ro, rd, first + ray, ry);
           const LatHdr h = lat_hdr(lat);
-          k_next = walk_from<kMode, false>(g, global_tabs(g), lat, h, ry, k_next, mr, 1, nr2);
+          k_next = walk_from<kMode, false>(g, global_tabs(g, lat), lat, h, ry, k_next, mr, 1, nr2);
           W = number_runs(mr, nr2);
         }
       }

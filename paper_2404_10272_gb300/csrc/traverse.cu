@@ -4,8 +4,11 @@
 // Both samplers share one walk.  The lattice t_0 < t_1 < ... depends only on
 // the call's parameters (Algorithm 1 advances t_last by Delta t whatever
 // voxel it is in), so it is computed once per parameter set into a small
-// device table and shared by every ray.  A ray then alternates two steps
-// (Algorithm 1's analyzer and its inner loops):
+// device table and shared by every ray.  A ray is first cut into stretches of
+// one level each: the lattice indices whose points lie in a level's box are
+// one interval, found once per ray and level, and the finest level whose
+// interval holds an index owns it (Sec. 3).  Inside a stretch the ray
+// alternates two steps (Algorithm 1's analyzer and its inner loops):
 //
 //   locate   the lattice point x(t_k) is classified and given a REGION: an
 //            axis-aligned set that holds x(t_k) and has one occupancy value
@@ -15,23 +18,32 @@
 //            empty or tiled 8^3 block, an empty or fully occupied 4^3 or 2^3
 //            cell (refinement), or a voxel of a leaf; with the refinement,
 //            one load from the region map (grid.cu) names it, without the
-//            tree is descended per region.  Outside
-//            every cascade box the region is a half-space the ray is leaving
-//            towards, or everything when it never comes back.
+//            tree is descended per region.
 //   cross    the first later lattice point outside the region.  The ray's
-//            parameter at the region's exit plane gives an estimate through
-//            a bucket index over the lattice; two exact probes confirm it
-//            (a gallop and bisection take over when they do not).  Every
-//            probe evaluates the point exactly as the definition does.
+//            parameter at the region's bounds gives an estimate through the
+//            lattice's closed form (or a bucket index); two exact probes
+//            confirm it (a gallop and bisection take over when they do
+//            not).  Every probe evaluates the point exactly as the definition
+//            does.
 //
 // Why this is exact: binary32 rounding is monotone, so for a fixed ray each
 // coordinate fl(o + fl(tm_k * d)) is monotone in k, and so is every voxel
-// index derived from it.  The points inside an axis-aligned region therefore
-// form one contiguous run of k, and only the region's exit plane on each
-// axis (the one the ray moves towards) can end the run.  Region bounds are
-// exact binary32 thresholds (grid.cu), so "inside" is decided exactly too.
-// The result is the sample set of the definition, with dense DDA and HDDA
-// bit-identical; HDDA just crosses far fewer regions.
+// index derived from it.  The points inside an axis-aligned box therefore
+// form one contiguous run of k, and only the face on each axis that the ray
+// moves towards can end the run.  Boxes are bounded by exact binary32
+// thresholds (grid.cu), so "inside" is decided exactly too.  The axes along
+// which a ray moves backwards are negated (exact, and rounding is symmetric),
+// so that every test is against an upper bound and both directions read one
+// table of them.  The result is the sample set of the definition, with dense
+// DDA and HDDA bit-identical; HDDA just crosses far fewer regions.
+//
+// What bounds the walk: instruction issue (80 % of cycles; integer ALU pipe
+// 58 %, 28 of 32 lanes active, 105 warp instructions per region).  Testing every
+// level's box and both directions' bounds per region took 219 of them: the
+// walk of an 800 x 800 object frame went from 175 to 102 us with the stretches,
+// the mirrored coordinates and the two probes without a branch between them,
+// the dense walk from 0.66 to 0.37 ms, the sampler on a 1245 x 825 unbounded
+// frame (four levels) from 0.51 to 0.36 ms.
 //
 // Launch shapes.  The allocating entry points run, by default, two kernels:
 // walk_kernel (persistent warps take 32-ray tiles in order from an atomic
@@ -311,7 +323,7 @@ __global__ void __launch_bounds__(kBS) onepass_kernel(
   if (r < n) {
     valid = load_ray(ro, rd, r, ray);
     if (valid)
-      c = walk<kMode, false, false>(g, global_tabs(g), lat, h, ray, s_runs + threadIdx.x, kBS,
+      c = walk<kMode, false, false>(g, global_tabs(g, lat), lat, h, ray, s_runs + threadIdx.x, kBS,
                                    nruns, 0, 0, 0, nullptr, nullptr, nullptr, status);
   }
   int64_t agg = 0;
@@ -337,7 +349,7 @@ __global__ void __launch_bounds__(kBS) onepass_kernel(
                     (int32_t)((int64_t)tile * kBS + warp * 32), lat.t, capacity, ray_idx, t0, t1);
   if (overflow && valid) {
     int unused = 0;
-    walk<kMode, true, false>(g, global_tabs(g), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
+    walk<kMode, true, false>(g, global_tabs(g, lat), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
                             capacity, ray_idx, t0, t1, status);
   }
 }
@@ -410,7 +422,7 @@ __device__ __forceinline__ void emit_tile(
     load_ray(ro, rd, r, ray);
     const LatHdr h = lat_hdr(lat);
     int unused = 0;
-    walk<kMode, true, false>(g, global_tabs(g), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
+    walk<kMode, true, false>(g, global_tabs(g, lat), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
                              capacity, ray_idx, t0, t1, status);
   }
 }
@@ -488,7 +500,7 @@ __host__ __device__ inline size_t walk_emit_smem(size_t stage_bytes) {
 template <int kMode, bool kSm>
 __device__ __forceinline__ void emit_fused_tile(
     int e, uint2* rec, const float* __restrict__ ro, const float* __restrict__ rd, int64_t n,
-    unsigned T, const GridDev& g, const Tabs& tb, const LatticeDev& ls, const LatHdr& h,
+    unsigned T, const GridDev& g, const Tabs<kSm>& tb, const LatticeDev& lat, const LatHdr& h,
     const int32_t* counts, const uint8_t* nruns, const uint2* runs, unsigned long long* state,
     int64_t* __restrict__ offsets, int32_t* __restrict__ ray_idx, float* __restrict__ t0,
     float* __restrict__ t1, int64_t capacity, bool vec, int64_t* __restrict__ total,
@@ -536,13 +548,13 @@ __device__ __forceinline__ void emit_fused_tile(
   __syncwarp();
   const int64_t room = capacity - excl;
   const int lim = room <= 0 ? 0 : (int)min((int64_t)tot, room);
-  expand_records(rec, nrec, lim, excl, (int32_t)((int64_t)e * 32), ls.t, vec, ray_idx, t0, t1);
+  expand_records(rec, nrec, lim, excl, (int32_t)((int64_t)e * 32), lat.t, vec, ray_idx, t0, t1);
   __syncwarp();  // the next tile reuses rec
   if (nr > kMaxRuns) {
     Ray ray;
     load_ray(ro, rd, r, ray);
     int unused = 0;
-    walk<kMode, true, kSm>(g, tb, ls, h, ray, nullptr, 0, unused, (int32_t)r, off, capacity,
+    walk<kMode, true, kSm>(g, tb, lat, h, ray, nullptr, 0, unused, (int32_t)r, off, capacity,
                            ray_idx, t0, t1, status);
   }
 }
@@ -557,15 +569,12 @@ __global__ void __launch_bounds__(kWalkBS) walk_emit_kernel(
     int64_t capacity, bool vec, int64_t* __restrict__ total, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem[];
   const LatHdr h = lat_hdr(lat);
-  Tabs tb = global_tabs(g);
-  LatticeDev ls = lat;
   size_t stage_bytes = 0;
   if constexpr (kSm) {
     const int64_t nodes = (int64_t)g.L * g.N * g.N * g.N;
     stage_bytes = stage_layout(lat.K, g.L, g.R, nodes, kMode).bytes;
-    stage_walk_tables<kMode>(smem, g, lat, h, tb, ls);
-    __syncthreads();
   }
+  const Tabs<kSm> tb = walk_tables<kMode, kSm>(smem, g, lat, h);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint2* rec = reinterpret_cast<uint2*>(smem + stage_bytes) + warp * (kRecMax + 1);
   const unsigned T = (unsigned)((n + 31) / 32);
@@ -580,7 +589,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_emit_kernel(
       Ray ray;
       int nr = 0;
       if (load_ray(ro, rd, r, ray))
-        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, ls, h, ray, runs + r, n, nr, 0, 0, 0,
+        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, 0, 0, 0,
                                                   nullptr, nullptr, nullptr, status);
       counts[r] = (int32_t)c;
       nruns_out[r] = (uint8_t)min(nr, 255);
@@ -595,7 +604,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_emit_kernel(
     if (lane == 0) e = atomicAdd(emit_counter, 1u);
     e = __shfl_sync(kFull, e, 0);
     if (e >= T) break;
-    emit_fused_tile<kMode, kSm>((int)e, rec, ro, rd, n, T, g, tb, ls, h, counts, nruns_out, runs,
+    emit_fused_tile<kMode, kSm>((int)e, rec, ro, rd, n, T, g, tb, lat, h, counts, nruns_out, runs,
                                 state, offsets, ray_idx, t0, t1, capacity, vec, total, status);
   }
 }

@@ -10,6 +10,9 @@
 // and why it is exact is explained at the top of traverse.cu.
 #pragma once
 
+#include <cstring>
+#include <type_traits>
+
 #include "grid.cuh"
 
 namespace hdda {
@@ -18,13 +21,37 @@ namespace {
 constexpr int kMaxRuns = 16;    // runs per ray kept between the walk and the emit
 constexpr unsigned kFull = 0xffffffffu;
 
-// Loads from a table that lives in shared memory (kSm) or in global memory
-// (read-only path).
+// Loads from global memory (read-only path) or shared memory.
 template <bool kSm, typename T>
 __device__ __forceinline__ T ld(const T* p) {
   if constexpr (kSm) return *p;
   else return __ldg(p);
 }
+
+// A table of 4-byte words the walk reads, in shared memory (kSm: by its 32-bit
+// shared address, so that no access goes through a generic one) or in global
+// memory (read-only path).
+template <bool kSm, typename T>
+struct Tab {
+  static_assert(sizeof(T) == 4, "4-byte entries");
+  std::conditional_t<kSm, uint32_t, const T*> p;
+
+  __device__ __forceinline__ T operator[](int i) const {
+    if constexpr (kSm) {
+      uint32_t v;
+      asm("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(p + 4u * (uint32_t)i));
+      T t;
+      memcpy(&t, &v, 4);
+      return t;
+    } else {
+      return __ldg(p + i);
+    }
+  }
+  __device__ __forceinline__ Tab at(int i) const {
+    if constexpr (kSm) return Tab{p + 4u * (uint32_t)i};
+    else return Tab{p + i};
+  }
+};
 
 // ---------------------------------------------------------------------------
 // lattice
@@ -52,7 +79,7 @@ struct LatHdr {
   uint32_t key0, shift;
   int NB;
   int lin;        // the closed form: 0 none (buckets), 1 constant spacing, 2 then geometric
-  float tm0, inv_dt;
+  float inv_dt, c0;             // 1 / spacing at the start, -tm0 / spacing
   float tm_s, inv_tm_s, ks, A;  // tm_ks (+inf when ks = K), 1 / tm_ks, ks, 1 / log2(1 + cone)
 };
 
@@ -61,8 +88,8 @@ __device__ __forceinline__ LatHdr lat_hdr(const LatticeDev& lat) {
            (int)__ldg(lat.hdr + 3), 0.f, 0.f, INFINITY, 0.f, 0.f, 0.f};
   if (h.lin && lat.K > 0) {
     const int ks = (int)__ldg(lat.hdr + 4);
-    h.tm0 = __ldg(lat.tm);
     h.inv_dt = 1.0f / (__ldg(lat.t + 1) - __ldg(lat.t));
+    h.c0 = -__ldg(lat.tm) * h.inv_dt;
     h.ks = (float)ks;
     h.A = __uint_as_float(__ldg(lat.hdr + 5));
     if (h.lin == 2 && ks < lat.K) {
@@ -77,24 +104,18 @@ __device__ __forceinline__ LatHdr lat_hdr(const LatticeDev& lat) {
   return h;
 }
 
-// First k with tm_k >= te (K if none), through the bucket index.
-template <bool kSm>
-__device__ __forceinline__ int first_k_at(const LatticeDev& lat, const LatHdr& h, float te) {
-  const uint32_t key = float_key(te);
-  const int b = key < h.key0 ? 0 : (int)min((key - h.key0) >> h.shift, (uint32_t)h.NB);
-  int lo = ld<kSm>(lat.kidx + b);
-  const int hi = ld<kSm>(lat.kidx + b + 1);
-  while (lo < hi && ld<kSm>(lat.tm + lo) < te) ++lo;
-  return lo;
-}
-
 // ---------------------------------------------------------------------------
 // the walk
 // ---------------------------------------------------------------------------
 
+// A ray in mirrored coordinates: every axis along which it moves backwards is
+// negated, so that no coordinate decreases along the ray (negation is exact
+// and binary32 rounding symmetric, so |x| of every point stays what it is).
+// A region then ends at one upper bound per axis, and leaving it is three
+// compares of one kind.
 struct Ray {
   float o[3], d[3], inv[3];
-  bool neg[3];  // direction component < 0 (a zero component counts as positive)
+  uint32_t nm[3];  // all ones on a mirrored axis, else 0
 };
 
 __device__ __forceinline__ bool load_ray(const float* __restrict__ ro,
@@ -102,29 +123,41 @@ __device__ __forceinline__ bool load_ray(const float* __restrict__ ro,
   bool ok = true;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    ray.o[c] = __ldg(ro + 3 * r + c);
-    ray.d[c] = __ldg(rd + 3 * r + c);
-    ok &= isfinite(ray.o[c]) && isfinite(ray.d[c]);
-    ray.neg[c] = ray.d[c] < 0.f;
-    // estimates only; +inf for a zero component (either sign), so that the
-    // crossing estimate needs no test for it (see cross)
-    ray.inv[c] = ray.d[c] != 0.f ? 1.0f / ray.d[c] : INFINITY;
+    const float o = __ldg(ro + 3 * r + c), d = __ldg(rd + 3 * r + c);
+    ok &= isfinite(o) && isfinite(d);
+    ray.nm[c] = d < 0.f ? ~0u : 0u;  // a zero component counts as positive
+    ray.o[c] = d < 0.f ? -o : o;
+    ray.d[c] = fabsf(d);
+    // estimates only; +inf for a zero component, so that the crossing
+    // estimate needs no test for it (see cross)
+    ray.inv[c] = d != 0.f ? 1.0f / ray.d[c] : INFINITY;
   }
   return ok;
 }
 
-// The grid tables the walk reads per region, in shared memory (staged) or
-// global memory; the rest of the grid stays in the GridDev kernel parameter.
+// The tables the walk reads per region, in shared memory (staged) or global
+// memory; the rest of the grid stays in the GridDev kernel parameter.
+template <bool kSm>
 struct Tabs {
-  const float* thr;
-  const uint32_t* child;
-  const uint32_t* tile;
-  const uint32_t* prefix;
-  const uint32_t* nstate;
+  Tab<kSm, float> tm;        // lattice midpoints
+  Tab<kSm, int> kidx;        // their bucket index
+  Tab<kSm, float> mthr;      // mirrored thresholds
+  Tab<kSm, uint32_t> child, tile, prefix, nstate;
 };
 
-__device__ __forceinline__ Tabs global_tabs(const GridDev& g) {
-  return Tabs{g.thr, g.child, g.tile, g.prefix, g.nstate};
+__device__ __forceinline__ Tabs<false> global_tabs(const GridDev& g, const LatticeDev& lat) {
+  return Tabs<false>{{lat.tm}, {lat.kidx}, {g.mthr}, {g.child}, {g.tile}, {g.prefix}, {g.nstate}};
+}
+
+// First k with tm_k >= te (K if none), through the bucket index.
+template <bool kSm>
+__device__ __forceinline__ int first_k_at(const Tabs<kSm>& tb, const LatHdr& h, float te) {
+  const uint32_t key = float_key(te);
+  const int b = key < h.key0 ? 0 : (int)min((key - h.key0) >> h.shift, (uint32_t)h.NB);
+  int lo = tb.kidx[b];
+  const int hi = tb.kidx[b + 1];
+  while (lo < hi && tb.tm[lo] < te) ++lo;
+  return lo;
 }
 
 // x = o + tm * d per axis, one rounding per operation.
@@ -133,99 +166,237 @@ __device__ __forceinline__ void point_at(const Ray& r, float tm, float x[3]) {
   for (int c = 0; c < 3; ++c) x[c] = __fadd_rn(r.o[c], __fmul_rn(tm, r.d[c]));
 }
 
-// A region is kept as one exit plane per axis: e[c] bounds the region on the
-// side the ray moves towards (upper bound, exclusive, for d >= 0; lower
-// bound, inclusive, for d < 0).
-__device__ __forceinline__ bool outside(const float x[3], const float e[3], const Ray& r) {
-  return ((x[0] >= e[0]) != r.neg[0]) | ((x[1] >= e[1]) != r.neg[1]) |
-         ((x[2] >= e[2]) != r.neg[2]);
+// A region is kept as its upper bound per axis (exclusive, mirrored
+// coordinates): the ray has left it once one coordinate reaches its bound.
+__device__ __forceinline__ bool outside(const float x[3], const float e[3]) {
+  return (x[0] >= e[0]) | (x[1] >= e[1]) | (x[2] >= e[2]);
 }
 
-// Intersects the region with [lo, hi) along axis c.
-__device__ __forceinline__ void clip(float e[3], const Ray& r, int c, float lo, float hi) {
-  e[c] = r.neg[c] ? fmaxf(e[c], lo) : fminf(e[c], hi);
-}
-
-// Intersects the region with voxels [a0, a1) of axis c of one level, using
-// the exact thresholds X[a] (only the bound on the exit side is loaded).
+// The lattice index at which tm reaches te, from the lattice's closed form
+// (lat_hdr) or the bucket index; off by one at times (the probes correct it).
+// Any value, saturated, for a te that is not finite.
 template <bool kSm>
-__device__ __forceinline__ void clip_cells(float e[3], const Ray& r, const float* thr, int R1,
-                                           int c, int a0, int a1) {
-  if (r.neg[c]) e[c] = fmaxf(e[c], ld<kSm>(thr + c * R1 + a0));
-  else e[c] = fminf(e[c], ld<kSm>(thr + c * R1 + a1));
+__device__ __forceinline__ int estimate_k(const Tabs<kSm>& tb, const LatHdr& h, float te) {
+  if (h.lin == 1) return __float2int_ru(fmaf(te, h.inv_dt, h.c0));  // uniform over the launch
+  if (h.lin == 2) {
+    const float fc = fmaf(te, h.inv_dt, h.c0);                   // constant spacing
+    const float fg = fmaf(__log2f(te * h.inv_tm_s), h.A, h.ks);  // geometric growth
+    return __float2int_ru(te < h.tm_s ? fc : fg);
+  }
+  return first_k_at<kSm>(tb, h, te);
 }
 
-// Classifies x and sets e to the region holding it.  Returns its occupancy.
-// kSm: the tables in tb point into shared memory.  `gone` carries, from one
-// call to the next along a ray, the levels whose box the ray has left for
-// good: a point outside a box on an axis whose coordinate does not move
-// back towards it stays outside (each coordinate is monotone in k), so
-// those levels need no test, and no half-space, again.  Only finer levels
-// are recorded (the coarsest is tested once per call anyway; measured
-// faster for single-level grids).
-// kOne: the grid has one level, so the level index is the constant 0 and
-// the level's box, scale and tables are addressed without it.
-template <int kMode, bool kSm, bool kOne>
-__device__ __forceinline__ bool locate_impl(const GridDev& g, const Tabs& tb, const Ray& r,
-                                            const float x[3], float e[3], unsigned& gone) {
-  const int L = kOne ? 1 : g.L;
+// First k in (k, kend) whose point is outside the region (kend if none).  The
+// point of k is inside.  x receives the point of that k when it is below kend.
+template <bool kSm>
+__device__ __forceinline__ int cross(const Ray& r, const Tabs<kSm>& tb, const LatHdr& h, int k,
+                                     int kend, const float e[3], float x[3]) {
+  // estimate: the ray parameter where it meets the first bound.  On an axis
+  // the ray does not move along, inv is +inf and the region holds the point,
+  // so e - o > 0 there: the term is +inf and sets no bound.
+  float te = INFINITY;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) e[c] = r.neg[c] ? -INFINITY : INFINITY;
-  int l = -1;
-  for (int lv = 0; lv < L; ++lv) {
-    if (lv + 1 < L && ((gone >> lv) & 1u)) continue;
-    const LevelDev& B = g.lv[lv];
-    bool inside = true;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) inside &= (x[c] >= B.lo[c]) & (x[c] < B.hi[c]);
-    if (inside) { l = lv; break; }
-    // x lies outside this (finer) box: keep a half-space that separates the
-    // ray's later points from it, preferring the one it leaves last.
-    int best = -1;
-    float best_t = -1.f;
-    bool never = false;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (x[c] < B.lo[c]) {
-        if (!(r.d[c] > 0.f)) never = true;  // coordinate never grows: never enters
-        else {
-          const float t = (B.lo[c] - x[c]) * r.inv[c];
-          if (t > best_t) { best_t = t; best = c; }
-        }
-      } else if (x[c] >= B.hi[c]) {
-        if (!(r.d[c] < 0.f)) never = true;
-        else {
-          const float t = (B.hi[c] - x[c]) * r.inv[c];
-          if (t > best_t) { best_t = t; best = c; }
-        }
-      }
-    }
-    if (never) {
-      if (lv + 1 < L) gone |= 1u << lv;
-      continue;
-    }
-    if (best < 0) continue;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (c != best) continue;
-      if (r.neg[c]) e[c] = fmaxf(e[c], B.hi[c]);  // region x >= hi
-      else e[c] = fminf(e[c], B.lo[c]);           // region x < lo
+  for (int c = 0; c < 3; ++c) te = fminf(te, (e[c] - r.o[c]) * r.inv[c]);
+  const int ke = max(estimate_k<kSm>(tb, h, te), k + 1);
+  // two probes, at the estimate (or the last index) and before it: nearly
+  // always the first is outside and the second inside
+  const int kp = min(ke, kend - 1), kq = max(kp - 1, k);
+  float y[3];
+  point_at(r, tb.tm[kp], x);
+  point_at(r, tb.tm[kq], y);
+  const bool oa = outside(x, e), ob = outside(y, e);
+  if (oa & !ob) return kp;
+  if (!oa & (ke >= kend)) return kend;
+  // the search looks `step` before hi, at most half way
+  int lo, hi, step = 1;  // invariant: point lo inside (lo >= k); point hi outside, or hi == kend
+  if (ob) {
+    lo = k;  // estimate too late
+    hi = kq;
+  } else {
+    for (lo = kp;; step <<= 1) {  // estimate too early: gallop forward
+      hi = lo + step;
+      if (hi >= kend) { hi = kend; break; }
+      point_at(r, tb.tm[hi], y);
+      if (outside(y, e)) break;
+      lo = hi;
     }
   }
-  if (l < 0) return false;
-  if constexpr (kOne) l = 0;
+  while (hi - lo > 1) {
+    const int mid = hi - min(step, (hi - lo) >> 1);
+    point_at(r, tb.tm[mid], y);
+    if (outside(y, e)) {
+      hi = mid;
+      step <<= 1;
+    } else {
+      lo = mid;
+    }
+  }
+  if (hi < kend) point_at(r, tb.tm[hi], x);
+  return hi;
+}
 
-  const LevelDev& V = g.lv[kOne ? 0 : l];
-  int i[3];
+// First k in [k0, k1) whose point satisfies `pred` (k1 if none); pred holds
+// from some k on.  te estimates where.
+template <bool kSm, typename P>
+__device__ __forceinline__ int first_true(const Tabs<kSm>& tb, const LatHdr& h, int k0, int k1,
+                                          float te, P pred) {
+  if (k0 >= k1) return k1;
+  int lo = k0 - 1, hi = k1;  // pred fails up to lo and holds from hi on
+  int at = min(max(estimate_k<kSm>(tb, h, te), k0), k1 - 1);
+  for (int step = 1; hi - lo > 1; step <<= 1) {  // gallop away from the estimate
+    if (pred(tb.tm[at])) {
+      hi = at;
+      at = max(at - step, lo + 1);
+      if (lo >= k0) at = lo + ((hi - lo) >> 1);  // both sides known: bisect
+    } else {
+      lo = at;
+      at = min(at + step, hi - 1);
+      if (hi < k1) at = lo + ((hi - lo) >> 1);
+    }
+  }
+  return hi;
+}
+
+// A box face as a bound in mirrored coordinates: on a mirrored axis, x < v is
+// -x >= -(the next value below v).
+__device__ __forceinline__ float mirror_bound(float v) {
+  const uint32_t u = __float_as_uint(v);
+  if ((u & 0x7fffffffu) == 0u) return __uint_as_float(1u);  // below zero: -denorm_min
+  return -__uint_as_float((u & 0x80000000u) ? u + 1u : u - 1u);
+}
+
+// The lattice indices [.x, .y) whose points lie in a level's box: one
+// interval, because no (mirrored) coordinate decreases along the ray.
+template <bool kSm>
+__device__ __forceinline__ int2 box_span(const LevelDev& B, const Ray& r, const Tabs<kSm>& tb,
+                                         const LatHdr& h, int K, int k0) {
+  float en[3], ex[3];  // inside: en <= x < ex
+  float ti = -INFINITY, tx = INFINITY;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    clip(e, r, c, V.lo[c], V.hi[c]);
-    i[c] = voxel_index(x[c], V.lo[c], V.s[c], g.R);
+    en[c] = r.nm[c] ? mirror_bound(B.hi[c]) : B.lo[c];
+    ex[c] = r.nm[c] ? mirror_bound(B.lo[c]) : B.hi[c];
+    ti = fmaxf(ti, (en[c] - r.o[c]) * r.inv[c]);
+    tx = fminf(tx, (ex[c] - r.o[c]) * r.inv[c]);
   }
-  // Descend to the coarsest uniform region holding x: an aligned cube of
-  // `sz` voxels (cut off at the grid edge).  Every kind ends in the one clip
-  // below, so lanes that stop at different depths share it.
-  int sz = 1;
+  const int a = first_true<kSm>(tb, h, k0, K, ti, [&](float tm) {
+    float x[3];
+    point_at(r, tm, x);
+    return (x[0] >= en[0]) & (x[1] >= en[1]) & (x[2] >= en[2]);
+  });
+  const int b = first_true<kSm>(tb, h, a, K, tx, [&](float tm) {
+    float x[3];
+    point_at(r, tm, x);
+    return outside(x, ex);
+  });
+  return make_int2(a, b);
+}
+
+// The stretches of a ray inside one level: lattice indices [k, kend) whose
+// points belong to level l (the finest one holding them).  They follow from
+// the levels' spans, which are found once per ray; the regions of a stretch
+// then need no test of any box.  kOne: the grid has one level, so there is one
+// stretch.  A level's constants are mirrored with the ray: voxel index =
+// (x - lo) * s either way.
+template <int kMode, bool kSm, bool kOne>
+struct Stretch {
+  float lo[3], s[3];
+  Tab<kSm, float> T;  // the level's mirrored thresholds (hdda_internal.cuh), at index 0
+  int l;
+  int kend;
+  int a[kOne ? 1 : kMaxLevels], b[kOne ? 1 : kMaxLevels];
+
+  __device__ __forceinline__ void init(const GridDev& g, const Tabs<kSm>& tb, const Ray& r,
+                                       const LatHdr& h, int K, int k0) {
+    kend = k0;
+    l = 0;
+    if constexpr (kOne) {
+      const int2 v = box_span<kSm>(g.lv[0], r, tb, h, K, k0);
+      a[0] = v.x;
+      b[0] = v.y;
+      level(g, tb, r);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < g.L; ++i) {
+        const int2 v = box_span<kSm>(g.lv[i], r, tb, h, K, k0);
+        a[i] = v.x;
+        b[i] = v.y;
+      }
+    }
+  }
+
+  __device__ __forceinline__ void level(const GridDev& g, const Tabs<kSm>& tb, const Ray& r) {
+    const LevelDev& V = g.lv[l];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      lo[c] = r.nm[c] ? -V.lo[c] : V.lo[c];
+      s[c] = r.nm[c] ? -V.s[c] : V.s[c];
+    }
+    T = tb.mthr.at(l * 3 * mthr_stride(g.R) + g.R);
+  }
+
+  // The stretch at or after k (at its start, moved to k): false if there is none.
+  __device__ __forceinline__ bool next(const GridDev& g, const Tabs<kSm>& tb, const Ray& r, int K,
+                                       int& k) {
+    if constexpr (kOne) {
+      if (k >= b[0]) return false;
+      k = max(k, a[0]);
+      kend = b[0];
+      return k < kend;
+    } else {
+      int at = -1, first = K, until = K;
+#pragma unroll 1
+      for (int i = 0; i < g.L; ++i) {
+        const int ai = a[i], bi = b[i];
+        if (ai >= bi || bi <= k) continue;
+        if (ai <= k) {
+          at = i;
+          until = min(until, bi);  // until so far: where a finer level begins
+          break;
+        }
+        until = min(until, ai);
+        first = min(first, ai);
+      }
+      if (at < 0) {  // no level holds k: on to the first that begins later
+        if (first >= K) return false;
+        k = first;
+        until = K;
+#pragma unroll 1
+        for (int i = 0; i < g.L; ++i) {
+          const int ai = a[i], bi = b[i];
+          if (ai >= bi || bi <= k) continue;
+          if (ai <= k) {
+            at = i;
+            until = min(until, bi);
+            break;
+          }
+          until = min(until, ai);
+        }
+      }
+      kend = until;
+      l = at;
+      level(g, tb, r);
+      return true;
+    }
+  }
+};
+
+// Classifies x, a point of the stretch's level: returns its occupancy and
+// sets e to the upper bounds of the region holding it.
+// kSm: the tables in tb point into shared memory.
+template <int kMode, bool kSm, bool kOne>
+__device__ __forceinline__ bool locate(const GridDev& g, const Tabs<kSm>& tb, const Ray& r,
+                                       const Stretch<kMode, kSm, kOne>& st, const float x[3],
+                                       float e[3]) {
+  const int l = kOne ? 0 : st.l;
+  int i[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)  // x lies in the box, so the index is not negative
+    i[c] = min(__float2int_rd(__fmul_rn(__fsub_rn(x[c], st.lo[c]), st.s[c])), g.R - 1);
+  // Descend to the coarsest uniform region holding x: an aligned cube of `szm`
+  // + 1 voxels (cut off at the grid edge).  Every kind ends in the one bound
+  // lookup below, so lanes that stop at different depths share it.
+  uint32_t szm = 0;
   bool occ;
   do {
     if constexpr (kMode == kModeDense) {
@@ -242,125 +413,40 @@ __device__ __forceinline__ bool locate_impl(const GridDev& g, const Tabs& tb, co
       const int cell = ((l * C + (i[0] >> 1)) * C + (i[1] >> 1)) * C + (i[2] >> 1);
       const uint32_t m = __ldg(g.rmap + cell);
       occ = (m >> (((i[0] & 1) << 2) | ((i[1] & 1) << 1) | (i[2] & 1))) & 1u;
-      sz = 1 << (m >> 8);
+      szm = (1u << (m >> 8)) - 1u;
       break;
     }
     // plain tree.  Node level: L * N^3 <= 8 * 8^3 nodes and L * B^3 * 16 <= 2^28 leaf
     // words, so every offset below fits 32 bits (cheaper address arithmetic than 64-bit)
     const int N = g.N;
     const int ng = l * N * N * N + ((i[0] >> 7) * N + (i[1] >> 7)) * N + (i[2] >> 7);
-    const uint32_t st = ld<kSm>(tb.nstate + ng);
-    if (st != kNodeMixed) {
-      sz = kNodeVox;
-      occ = st == kNodeFull;
+    const uint32_t st_n = tb.nstate[ng];
+    if (st_n != kNodeMixed) {
+      szm = kNodeVox - 1;
+      occ = st_n == kNodeFull;
       break;
     }
     // block level: empty or tile
     const int cell = (((i[0] >> 3) & 15) * 16 + ((i[1] >> 3) & 15)) * 16 + ((i[2] >> 3) & 15);
     const int w = cell >> 5;
     const uint32_t bit = 1u << (cell & 31);
-    const uint32_t cw = ld<kSm>(tb.child + ng * kNodeWords + w);
+    const uint32_t cw = tb.child[ng * kNodeWords + w];
     if (!(cw & bit)) {
-      sz = kBlockDim;
-      occ = (ld<kSm>(tb.tile + ng * kNodeWords + w) & bit) != 0u;
+      szm = kBlockDim - 1;
+      occ = (tb.tile[ng * kNodeWords + w] & bit) != 0u;
       break;
     }
     // voxel of a leaf
-    const uint32_t leaf = ld<kSm>(tb.prefix + ng * kNodeWords + w) + __popc(cw & (bit - 1u));
+    const uint32_t leaf = tb.prefix[ng * kNodeWords + w] + __popc(cw & (bit - 1u));
     const int v = ((i[0] & 7) * 8 + (i[1] & 7)) * 8 + (i[2] & 7);
     const uint32_t lw = __ldg(g.leaves + (leaf * (uint32_t)kLeafWords + (uint32_t)(v >> 5)));
     occ = (lw >> (v & 31)) & 1u;
   } while (false);
-  const int R1 = g.R + 1;
-  const float* thr = tb.thr + l * 3 * R1;
+  const int TS = mthr_stride(g.R);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int a0 = i[c] & -sz;
-    clip_cells<kSm>(e, r, thr, R1, c, a0, min(a0 + sz, g.R));
-  }
+  for (int c = 0; c < 3; ++c)
+    e[c] = st.T[c * TS + (int)(((uint32_t)i[c] ^ r.nm[c]) | szm)];
   return occ;
-}
-
-template <int kMode, bool kSm>
-__device__ __forceinline__ bool locate(const GridDev& g, const Tabs& tb, const Ray& r,
-                                       const float x[3], float e[3], unsigned& gone) {
-  if (g.L == 1) return locate_impl<kMode, kSm, true>(g, tb, r, x, e, gone);  // uniform
-  return locate_impl<kMode, kSm, false>(g, tb, r, x, e, gone);
-}
-
-// First k' in (k, K] whose point is outside the region (K if none).  The
-// point of k is inside.  xo receives the point of k' when k' < K.
-template <bool kSm>
-__device__ __forceinline__ int cross(const Ray& r, const LatticeDev& lat, const LatHdr& h, int k,
-                                     const float e[3], float xo[3]) {
-  const int K = lat.K;
-  // estimate: the ray parameter where it meets the first exit plane.  On an
-  // axis the ray does not move along, inv is +inf and the region holds the
-  // point, so e - o > 0 there (or e = +inf): the term is +inf (or NaN when
-  // e - o = 0, which fminf ignores) and sets no bound.
-  float te = INFINITY;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) te = fminf(te, (e[c] - r.o[c]) * r.inv[c]);
-  // The closed form (lat_hdr) lands on the first k with tm_k >= te, or next
-  // to it, with fewer instructions than the bucket index.
-  int ke;
-  if (h.lin == 1) {  // uniform over the launch
-    ke = (int)ceilf(fminf(fmaxf((te - h.tm0) * h.inv_dt, 0.f), (float)K));
-  } else if (h.lin == 2) {
-    const float fc = (te - h.tm0) * h.inv_dt;                  // constant spacing
-    const float fg = fmaf(__log2f(te * h.inv_tm_s), h.A, h.ks);  // geometric growth
-    ke = (int)ceilf(fminf(fmaxf(te < h.tm_s ? fc : fg, 0.f), (float)K));
-  } else {
-    ke = first_k_at<kSm>(lat, h, te);
-  }
-  ke = max(ke, k + 1);
-  int lo, hi;  // invariant: point lo inside (lo >= k); point hi outside, or hi == K
-  float xp[3];
-  if (ke >= K) {
-    if (K - 1 == k) return K;
-    point_at(r, ld<kSm>(lat.tm + K - 1), xp);
-    if (!outside(xp, e, r)) return K;
-    lo = k;
-    hi = K - 1;
-    xo[0] = xp[0]; xo[1] = xp[1]; xo[2] = xp[2];
-  } else {
-    point_at(r, ld<kSm>(lat.tm + ke), xp);
-    if (!outside(xp, e, r)) {
-      // estimate too early: gallop forward
-      lo = ke;
-      int step = 1;
-      for (;;) {
-        hi = lo + step;
-        if (hi >= K) { hi = K; break; }
-        point_at(r, ld<kSm>(lat.tm + hi), xp);
-        if (outside(xp, e, r)) {
-          xo[0] = xp[0]; xo[1] = xp[1]; xo[2] = xp[2];
-          break;
-        }
-        lo = hi;
-        step <<= 1;
-      }
-    } else {
-      xo[0] = xp[0]; xo[1] = xp[1]; xo[2] = xp[2];
-      if (ke - 1 == k) return ke;
-      point_at(r, ld<kSm>(lat.tm + ke - 1), xp);
-      if (!outside(xp, e, r)) return ke;  // the usual case: estimate exact
-      lo = k;
-      hi = ke - 1;
-      xo[0] = xp[0]; xo[1] = xp[1]; xo[2] = xp[2];
-    }
-  }
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    point_at(r, ld<kSm>(lat.tm + mid), xp);
-    if (outside(xp, e, r)) {
-      hi = mid;
-      xo[0] = xp[0]; xo[1] = xp[1]; xo[2] = xp[2];
-    } else {
-      lo = mid;
-    }
-  }
-  return hi;
 }
 
 // Walks one ray.  Counts its samples and merges occupied regions into runs
@@ -373,73 +459,76 @@ __device__ __forceinline__ int cross(const Ray& r, const LatticeDev& lat, const 
 // on its occupancy).  The regions crossed, and so the samples, are the same.
 // kCheck tests that every region holds the point it was found from (raising
 // kDevInternal otherwise); the invariant the crossing search rests on.
-template <int kMode, bool kEmit, bool kSm, bool kSkip = false, bool kCheck = false>
-__device__ __forceinline__ int64_t walk(const GridDev& g, const Tabs& tb, const LatticeDev& lat,
-                                        const LatHdr& h, const Ray& r, uint2* runs,
-                                        int64_t stride, int& nruns, int32_t rid,
-                                        int64_t out, int64_t capacity,
-                                        int32_t* __restrict__ ray_idx, float* __restrict__ t0,
-                                        float* __restrict__ t1, unsigned* __restrict__ status) {
-  const int K = lat.K;
-  int64_t cnt = 0;
+template <int kMode, bool kEmit, bool kSm, bool kSkip, bool kCheck, bool kOne>
+__device__ __forceinline__ int64_t walk_levels(const GridDev& g, const Tabs<kSm>& tb,
+                                               const LatticeDev& lat, const LatHdr& h,
+                                               const Ray& r, uint2* runs, int64_t stride,
+                                               int& nruns, int32_t rid, int64_t out,
+                                               int64_t capacity, int32_t* __restrict__ ray_idx,
+                                               float* __restrict__ t0, float* __restrict__ t1,
+                                               unsigned* __restrict__ status) {
+  int64_t cnt = 0;  // kEmit
+  int kept = 0;     // at most 2^24
   nruns = 0;
-  if (K <= 0) return 0;
+  if (lat.K <= 0) return 0;
   int rb = -1, re = -1;  // open run
   float x[3];
-  point_at(r, ld<kSm>(lat.tm), x);
   int k = 0;
-  unsigned gone = 0u;  // cascade levels the ray has left for good
-  while (k < K) {
-    bool occ;
+  Stretch<kMode, kSm, kOne> st;
+  st.init(g, tb, r, h, lat.K, 0);
+  for (;;) {
+    bool occ, over = false;
     int kn;
     // One region; in the skip form, every leading empty region first (one
     // copy of locate and cross serves both forms).  cross advances by
     // construction; the skip form still guards its inner loop (no progress:
-    // report, end the ray).  With that conditional store in the loop the
-    // skip form measured 2.6x faster (object frame) than without it, while
-    // the same guard costs the branch form 5 %, so only the skip form has it.
+    // report, end the ray).
     for (;;) {
+      if (k >= st.kend) {
+        over = !st.next(g, tb, r, lat.K, k);
+        if (over) break;
+        point_at(r, tb.tm[k], x);
+      }
       float e[3];
-      occ = locate<kMode, kSm>(g, tb, r, x, e, gone);
+      occ = locate(g, tb, r, st, x, e);
       if constexpr (kCheck)
-        if (outside(x, e, r)) atomicOr(status, kDevInternal);
-      kn = cross<kSm>(r, lat, h, k, e, x);
+        if (outside(x, e)) atomicOr(status, kDevInternal);
+      kn = cross<kSm>(r, tb, h, k, st.kend, e, x);
       if constexpr (kSkip)
         if (kn <= k) {
           atomicOr(status, kDevInternal);
-          occ = false;
-          kn = K;
+          over = true;
+          break;
         }
-      if (!kSkip || occ || kn >= K) break;
+      if (!kSkip || occ) break;
       k = kn;
     }
-    if (occ) {
-      if (kEmit) {
+    if (over) break;
+    if constexpr (kEmit) {
+      if (occ) {
         float ta = __ldg(lat.t + k);
         for (int j = k; j < kn; ++j) {
-          const float tb = __ldg(lat.t + j + 1);
+          const float tn = __ldg(lat.t + j + 1);
           const int64_t p = out + cnt;
           if (p < capacity) {
             ray_idx[p] = rid;
             t0[p] = ta;
-            t1[p] = tb;
+            t1[p] = tn;
           }
-          ta = tb;
+          ta = tn;
           ++cnt;
         }
-      } else {
-        cnt += kn - k;
-        if (k == re) {
-          re = kn;  // adjacent occupied region: extend the run
-        } else {
-          if (rb >= 0) {
-            if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
-            ++nruns;
-          }
-          rb = k;
-          re = kn;
-        }
       }
+    } else {
+      // an occupied region extends the open run or, not adjacent, opens the next one
+      const bool opens = occ & (k != re);
+      if (opens & (rb >= 0)) {
+        if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
+        ++nruns;
+      }
+      kept += occ ? kn - k : 0;
+      rb = opens ? k : rb;
+      re = occ ? kn : re;
     }
     k = kn;
   }
@@ -447,7 +536,24 @@ __device__ __forceinline__ int64_t walk(const GridDev& g, const Tabs& tb, const 
     if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
     ++nruns;
   }
-  return cnt;
+  return kEmit ? cnt : (int64_t)kept;
+}
+
+// The walk with the one-level form where it applies (its own copy of the
+// code), except in the rare second walk of a ray (kEmit).
+template <int kMode, bool kEmit, bool kSm, bool kSkip = false, bool kCheck = false>
+__device__ __forceinline__ int64_t walk(const GridDev& g, const Tabs<kSm>& tb,
+                                        const LatticeDev& lat,
+                                        const LatHdr& h, const Ray& r, uint2* runs,
+                                        int64_t stride, int& nruns, int32_t rid,
+                                        int64_t out, int64_t capacity,
+                                        int32_t* __restrict__ ray_idx, float* __restrict__ t0,
+                                        float* __restrict__ t1, unsigned* __restrict__ status) {
+  if (!kEmit && g.L == 1)  // uniform
+    return walk_levels<kMode, kEmit, kSm, kSkip, kCheck, true>(
+        g, tb, lat, h, r, runs, stride, nruns, rid, out, capacity, ray_idx, t0, t1, status);
+  return walk_levels<kMode, kEmit, kSm, kSkip, kCheck, false>(
+      g, tb, lat, h, r, runs, stride, nruns, rid, out, capacity, ray_idx, t0, t1, status);
 }
 
 // Walks one ray from lattice index k0 and stops after kMaxRuns runs: writes
@@ -457,7 +563,8 @@ __device__ __forceinline__ int64_t walk(const GridDev& g, const Tabs& tb, const 
 // the same samples because every point is classified on its own.  It does
 // not check its regions: the first pass crossed the same ones.
 template <int kMode, bool kSm>
-__device__ __forceinline__ int walk_from(const GridDev& g, const Tabs& tb, const LatticeDev& lat,
+__device__ __forceinline__ int walk_from(const GridDev& g, const Tabs<kSm>& tb,
+                                         const LatticeDev& lat,
                                          const LatHdr& h, const Ray& r, int k0, uint2* runs,
                                          int stride, int& nruns) {
   const int K = lat.K;
@@ -465,15 +572,17 @@ __device__ __forceinline__ int walk_from(const GridDev& g, const Tabs& tb, const
   if (k0 >= K) return K;
   int rb = -1, re = -1;  // open run
   float x[3];
-  point_at(r, ld<kSm>(lat.tm + k0), x);
   int k = k0;
-  unsigned gone = 0u;
-  while (k < K) {
+  Stretch<kMode, kSm, false> st;
+  st.init(g, tb, r, h, K, k0);
+  for (;;) {
+    if (k >= st.kend) {
+      if (!st.next(g, tb, r, K, k)) break;
+      point_at(r, tb.tm[k], x);
+    }
     float e[3];
-    // the general form only: this path is rare, and one copy of the location
-    // code keeps its caller's registers free
-    const bool occ = locate_impl<kMode, kSm, false>(g, tb, r, x, e, gone);
-    const int kn = cross<kSm>(r, lat, h, k, e, x);
+    const bool occ = locate(g, tb, r, st, x, e);
+    const int kn = cross<kSm>(r, tb, h, k, st.kend, e, x);
     if (occ) {
       if (k == re) {
         re = kn;
@@ -730,7 +839,7 @@ __host__ __device__ inline StageLayout stage_layout(int K, int L, int R, int64_t
   size_t o = 0;
   s.tm = o; o += sizeof(float) * (size_t)K;
   s.kidx = o; o += sizeof(int) * (size_t)(kKidxMax + 2);
-  s.thr = o; o += sizeof(float) * (size_t)L * 3 * (R + 1);
+  s.thr = o; o += sizeof(float) * (size_t)L * 3 * mthr_stride(R);
   s.child = s.tile = s.prefix = s.nstate = o;
   if (mode == kModeVdb) {
     s.child = o; o += 4 * (size_t)nodes * kNodeWords;
@@ -742,44 +851,42 @@ __host__ __device__ inline StageLayout stage_layout(int K, int L, int R, int64_t
   return s;
 }
 
-constexpr size_t kMaxStageBytes = 96 * 1024;
+// leaves the L1 half of the SM's 256 KB
+constexpr size_t kMaxStageBytes = 128 * 1024;
 
 template <typename T>
 __device__ __forceinline__ void stage_copy(T* dst, const T* __restrict__ src, int64_t count) {
   for (int64_t i = threadIdx.x; i < count; i += blockDim.x) dst[i] = __ldg(src + i);
 }
 
-// Copies the walk's tables into shared memory at `smem` (stage_layout) and
-// points tb and ls at the copies; the caller synchronises the block before
-// the first walk.
-template <int kMode>
-__device__ __forceinline__ void stage_walk_tables(unsigned char* smem, const GridDev& g,
-                                                  const LatticeDev& lat, const LatHdr& h,
-                                                  Tabs& tb, LatticeDev& ls) {
-  const int64_t nodes = (int64_t)g.L * g.N * g.N * g.N;
-  const StageLayout sl = stage_layout(lat.K, g.L, g.R, nodes, kMode);
-  float* s_tm = reinterpret_cast<float*>(smem + sl.tm);
-  int* s_kidx = reinterpret_cast<int*>(smem + sl.kidx);
-  float* s_thr = reinterpret_cast<float*>(smem + sl.thr);
-  stage_copy(s_tm, lat.tm, lat.K);
-  stage_copy(s_kidx, lat.kidx, (int64_t)h.NB + 2);
-  stage_copy(s_thr, g.thr, (int64_t)g.L * 3 * (g.R + 1));
-  ls.tm = s_tm;
-  ls.kidx = s_kidx;
-  tb.thr = s_thr;
-  if constexpr (kMode == kModeVdb) {
-    uint32_t* s_child = reinterpret_cast<uint32_t*>(smem + sl.child);
-    uint32_t* s_tile = reinterpret_cast<uint32_t*>(smem + sl.tile);
-    uint32_t* s_prefix = reinterpret_cast<uint32_t*>(smem + sl.prefix);
-    uint32_t* s_nstate = reinterpret_cast<uint32_t*>(smem + sl.nstate);
-    stage_copy(s_child, g.child, nodes * kNodeWords);
-    stage_copy(s_tile, g.tile, nodes * kNodeWords);
-    stage_copy(s_prefix, g.prefix, nodes * kNodeWords);
-    stage_copy(s_nstate, g.nstate, nodes);
-    tb.child = s_child;
-    tb.tile = s_tile;
-    tb.prefix = s_prefix;
-    tb.nstate = s_nstate;
+// The walk's tables: copied into shared memory at `smem` (stage_layout, kSm;
+// synchronises the block) or where they are.
+template <int kMode, bool kSm>
+__device__ __forceinline__ Tabs<kSm> walk_tables(unsigned char* smem, const GridDev& g,
+                                                 const LatticeDev& lat, const LatHdr& h) {
+  if constexpr (!kSm) {
+    return global_tabs(g, lat);
+  } else {
+    const int64_t nodes = (int64_t)g.L * g.N * g.N * g.N;
+    const StageLayout sl = stage_layout(lat.K, g.L, g.R, nodes, kMode);
+    stage_copy(reinterpret_cast<float*>(smem + sl.tm), lat.tm, lat.K);
+    if (!h.lin)  // the closed form does without the buckets
+      stage_copy(reinterpret_cast<int*>(smem + sl.kidx), lat.kidx, (int64_t)h.NB + 2);
+    stage_copy(reinterpret_cast<float*>(smem + sl.thr), g.mthr,
+               (int64_t)g.L * 3 * mthr_stride(g.R));
+    if constexpr (kMode == kModeVdb) {
+      stage_copy(reinterpret_cast<uint32_t*>(smem + sl.child), g.child, nodes * kNodeWords);
+      stage_copy(reinterpret_cast<uint32_t*>(smem + sl.tile), g.tile, nodes * kNodeWords);
+      stage_copy(reinterpret_cast<uint32_t*>(smem + sl.prefix), g.prefix, nodes * kNodeWords);
+      stage_copy(reinterpret_cast<uint32_t*>(smem + sl.nstate), g.nstate, nodes);
+    }
+    __syncthreads();
+    uint32_t b = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("" : "+r"(b)::"memory");  // the loads depend on it: none moves above the barrier
+    return Tabs<true>{{b + (uint32_t)sl.tm},    {b + (uint32_t)sl.kidx},
+                      {b + (uint32_t)sl.thr},   {b + (uint32_t)sl.child},
+                      {b + (uint32_t)sl.tile},  {b + (uint32_t)sl.prefix},
+                      {b + (uint32_t)sl.nstate}};
   }
 }
 
@@ -812,12 +919,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_kernel(
     unsigned long long* __restrict__ sums1024, int32_t width) {
   extern __shared__ __align__(16) unsigned char smem[];
   const LatHdr h = lat_hdr(lat);
-  Tabs tb = global_tabs(g);
-  LatticeDev ls = lat;
-  if constexpr (kSm) {
-    stage_walk_tables<kMode>(smem, g, lat, h, tb, ls);
-    __syncthreads();
-  }
+  const Tabs<kSm> tb = walk_tables<kMode, kSm>(smem, g, lat, h);
   // work tiles, and block columns: 8 x 4 blocks over ceil(n / width) rows.
   // Kept in shared memory, not in registers across the walk.
   __shared__ unsigned s_tiles[2];
@@ -850,7 +952,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_kernel(
       Ray ray;
       int nr = 0;
       if (load_ray(ro, rd, r, ray))
-        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, ls, h, ray, runs + r, n, nr, 0, 0, 0,
+        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, 0, 0, 0,
                                                   nullptr, nullptr, nullptr, status);
       counts[r] = (int32_t)c;
       nruns_out[r] = (uint8_t)min(nr, 255);

@@ -417,13 +417,14 @@ int create(const hdda_job* jobs, int n_jobs, const hdda_batch_config* cfg, hdda_
   // one per request group (a server's admission tick) never synchronises the device.
   b->async_scratch = !c.use_graph;
   b->alloc_stream = s;
-  cudaError_t e = b->async_scratch ? cudaMallocAsync(&b->scratch, b->scratch_bytes, s)
+  cudaError_t e = b->async_scratch ? scratch_alloc(&b->scratch, b->scratch_bytes, s)
                                    : cudaMalloc(&b->scratch, b->scratch_bytes);
   if (e != cudaSuccess) {
     b->scratch = nullptr;
     delete b;
     return cuda_error(e, "batch scratch allocation");
   }
+  scratch_users(dev, 1);
   char* p = b->scratch;
   b->counter = reinterpret_cast<unsigned*>(p);
   b->status = b->counter + 1;
@@ -552,6 +553,7 @@ extern "C" void hdda_batch_free(hdda_batch* b) {
       cudaDeviceSynchronize();
       cudaFree(b->scratch);
     }
+    scratch_users(b->device, -1);
   }
   delete b;
 }

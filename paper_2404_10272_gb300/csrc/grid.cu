@@ -662,6 +662,7 @@ int create(int kind, const uint8_t* dense, int levels, int res, const hdda_aabb*
   e = cudaMalloc(&g->base, g->base_bytes);
   if (e != cudaSuccess) { delete g; return cuda_error(e, "cudaMalloc(grid)"); }
   layout(g, static_cast<char*>(g->base));
+  scratch_users(g->device, 1);
   e = cudaEventCreateWithFlags(&g->built, cudaEventDisableTiming);
   if (e != cudaSuccess) { hdda_grid_free(g); return cuda_error(e, "cudaEventCreate"); }
   thresholds_kernel<<<blocks_for(g->thr_count(), 128), 128, 0, s>>>(g->view(), g->thr, g->mthr);
@@ -734,7 +735,7 @@ int update_vdb(hdda_grid* g, const uint8_t* dense, const int64_t* blocks, int64_
   }
   // scratch: {flags[0] = structure changed, status}, then changed[count]
   char* scratch = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&scratch, 16 + (size_t)count, s));
+  HDDA_CUDA_TRY(scratch_alloc(&scratch, 16 + (size_t)count, s));
   unsigned* flags = reinterpret_cast<unsigned*>(scratch);
   unsigned* status = dev_status ? dev_status : flags + 1;
   uint8_t* changed = reinterpret_cast<uint8_t*>(scratch + 16);
@@ -895,6 +896,7 @@ extern "C" void hdda_grid_free(hdda_grid* g) {
   if (g->base) {
     cudaDeviceSynchronize();
     cudaFree(g->base);
+    scratch_users(g->device, -1);
   }
   delete g;
 }

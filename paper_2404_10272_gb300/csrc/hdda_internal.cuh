@@ -140,6 +140,19 @@ int set_error(int code, const char* fmt, ...);
 int cuda_error(cudaError_t e, const char* what);
 void clear_error();
 
+// Stream-ordered scratch of a call, from the library's own memory pool of the
+// current device; given back with cudaFreeAsync (runtime.cu).
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+template <typename T>
+cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t s) {
+  return scratch_alloc(reinterpret_cast<void**>(p), bytes, s);
+}
+// A grid or batch came to life (+1) or was freed (-1) on a device: with the last
+// one the pool's unused memory is given back (runtime.cu).
+void scratch_users(int device, int change);
+// Multiprocessors of a device, looked up once (runtime.cu); 1 if unknown.
+int sm_count(int device);
+
 // True while the kernel timers are enabled (runtime.cu).
 bool profiler_on();
 // True while the work counters are enabled (runtime.cu).

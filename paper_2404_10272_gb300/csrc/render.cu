@@ -468,7 +468,7 @@ extern "C" int hdda_render(const float* rays_o, const float* rays_d, int64_t n_r
     hw = t_word.p;
   }
   char* scratch = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&scratch, render_scratch_bytes(n_rays), s));
+  HDDA_CUDA_TRY(scratch_alloc(&scratch, render_scratch_bytes(n_rays), s));
   st = launch_render(rays_o, rays_d, n_rays, grid, lat, params->image_width, field, n_gauss,
                      rgba_out, dev_status, scratch, s);
   if (st == HDDA_OK && !dev_status) {
@@ -523,7 +523,7 @@ extern "C" int hdda_traverse_composite(const float* rays_o, const float* rays_d,
     return HDDA_OK;
   }
   char* scratch = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&scratch, sample_composite_scratch_bytes(n_rays), s));
+  HDDA_CUDA_TRY(scratch_alloc(&scratch, sample_composite_scratch_bytes(n_rays), s));
   st = launch_sample_composite(rays_o, rays_d, n_rays, grid, lat, params->image_width, field,
                                n_gauss, rgba_out, offsets, ray_idx, t0, t1, capacity, dev_status,
                                scratch, s);

@@ -29,6 +29,82 @@ int cuda_error(cudaError_t e, const char* what) {
 void clear_error() { g_last_error[0] = '\0'; }
 
 // ---------------------------------------------------------------------------
+// scratch memory
+// ---------------------------------------------------------------------------
+// A call's scratch (about 134 bytes per ray) comes from a stream-ordered pool
+// of the library's own, one per device, that keeps up to kPoolKeep bytes of
+// unused memory across synchronisations.  The device's default pool keeps none
+// (that is its owner's to choose), so that every call after a synchronisation
+// mapped its scratch anew: 300 us for a 9,216-ray frame whose kernels take 75,
+// and 0.65 against 0.25 ms for an 800 x 800 sampler call waited for.  The bound holds a
+// call of seven million rays, or several smaller ones in flight at once; more
+// is given back at the next synchronisation, and all of it with the device's
+// last grid and batch.
+namespace {
+constexpr int kMaxPoolDevices = 64;
+constexpr uint64_t kPoolKeep = 1ull << 30;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[kMaxPoolDevices] = {};
+int64_t g_pool_users[kMaxPoolDevices] = {};
+std::atomic<int> g_sms[kMaxPoolDevices] = {};
+
+cudaError_t pool_of(int dev, cudaMemPool_t* out) {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pools[dev]) {
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = kPoolKeep;
+    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(pool);
+      return e;
+    }
+    g_pools[dev] = pool;
+  }
+  *out = g_pools[dev];
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxPoolDevices) return cudaMallocAsync(p, bytes, s);
+  cudaMemPool_t pool = nullptr;
+  e = pool_of(dev, &pool);
+  if (e != cudaSuccess) return e;
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+void scratch_users(int device, int change) {
+  if (device < 0 || device >= kMaxPoolDevices) return;
+  cudaMemPool_t pool = nullptr;
+  // made here, where memory is allocated anyway, and not first inside a stream capture
+  if (change > 0 && pool_of(device, &pool) != cudaSuccess) cudaGetLastError();
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  g_pool_users[device] += change;
+  if (g_pool_users[device] == 0 && g_pools[device]) cudaMemPoolTrimTo(g_pools[device], 0);
+}
+
+int sm_count(int device) {
+  const bool known = device >= 0 && device < kMaxPoolDevices;
+  int n = known ? g_sms[device].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n < 1)
+    return 1;
+  if (known) g_sms[device].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// ---------------------------------------------------------------------------
 // profiler
 // ---------------------------------------------------------------------------
 namespace {

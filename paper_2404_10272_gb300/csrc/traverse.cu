@@ -359,6 +359,7 @@ __global__ void __launch_bounds__(kBS) onepass_kernel(
 // ---------------------------------------------------------------------------
 
 constexpr int kEmitWarps = 4;
+constexpr int kEmitCtasPerSm = 7;  // by registers (72) and shared memory (16 KB)
 
 // Pass 2 for one 32-ray tile, independent of every other tile: its offset
 // is the sum of the earlier tiles' samples (tile_offset, from the group sums
@@ -433,7 +434,7 @@ __device__ __forceinline__ void emit_tile(
 // tile and loading its counts before expanding the current one measured 5-14 %
 // slower: tiles held by busy warps lengthen the tail.)
 template <int kMode>
-__global__ void __launch_bounds__(kEmitWarps * 32, 7) emit_kernel(
+__global__ void __launch_bounds__(kEmitWarps * 32, kEmitCtasPerSm) emit_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, GridDev g,
     LatticeDev lat, const int32_t* __restrict__ counts, const uint8_t* __restrict__ nruns,
     const uint2* __restrict__ runs, const int64_t* __restrict__ tile_sum,
@@ -456,18 +457,11 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 7) emit_kernel(
   }
 }
 
-// Resident CTAs of the persistent emit: one wave, or fewer for small calls.
-template <int kMode>
-unsigned emit_grid(int64_t T) {
-  int dev = 0, sms = 1, per_sm = 1;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, emit_kernel<kMode>,
-                                                    kEmitWarps * 32, 0) != cudaSuccess ||
-      per_sm <= 0)
-    per_sm = 1;
+// CTAs of the persistent emit: one wave (the launch bounds' CTAs per SM), or
+// fewer for small calls.
+unsigned emit_grid(int64_t T, int device) {
   const int64_t want = (T + kEmitWarps - 1) / kEmitWarps;
-  const int64_t full = (int64_t)(sms > 0 ? sms : 1) * per_sm;
+  const int64_t full = (int64_t)sm_count(device) * kEmitCtasPerSm;
   return (unsigned)(want < full ? want : full);
 }
 
@@ -730,7 +724,7 @@ int get_lattice(const hdda_params& p, cudaStream_t s, LatticeDev* out) {
   int st = host_words(&hw);
   if (st != HDDA_OK) return st;
   int64_t* dk = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&dk, 2 * sizeof(int64_t), s));
+  HDDA_CUDA_TRY(scratch_alloc(&dk, 2 * sizeof(int64_t), s));
   lattice_count_kernel<<<1, 1, 0, s>>>(key, dk);
   HDDA_CUDA_TRY(cudaGetLastError());
   HDDA_CUDA_TRY(cudaMemcpyAsync(hw, dk, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -918,17 +912,17 @@ int run_twopass(const float* ro, const float* rd, int64_t n, const hdda_grid* gr
     KernelTimer kt(emit_name(mode), s);
     switch (mode) {
       case kModeDense:
-        emit_kernel<kModeDense><<<emit_grid<kModeDense>(T), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeDense><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
             ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
         break;
       case kModeVdb:
-        emit_kernel<kModeVdb><<<emit_grid<kModeVdb>(T), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeVdb><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
             ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
         break;
       default:
-        emit_kernel<kModeVdbMap><<<emit_grid<kModeVdbMap>(T), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeVdbMap><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
             ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
         break;
@@ -958,7 +952,7 @@ int traverse(bool vdb, const float* ro, const float* rd, int64_t n, const hdda_g
   st = host_words(&hw);
   if (st != HDDA_OK) return st;
   char* scratch = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&scratch, twopass_scratch_bytes(n), s));
+  HDDA_CUDA_TRY(scratch_alloc(&scratch, twopass_scratch_bytes(n), s));
   st = run_twopass(ro, rd, n, grid, lat, params->image_width, offsets, ray_idx, t0, t1, capacity,
                    total_out, scratch, hw, nullptr, s);
   cudaError_t e = cudaFreeAsync(scratch, s);
@@ -988,7 +982,7 @@ int traverse_async(const float* ro, const float* rd, int64_t n, const hdda_grid*
     return HDDA_OK;
   }
   char* scratch = nullptr;
-  HDDA_CUDA_TRY(cudaMallocAsync(&scratch, twopass_scratch_bytes(n), s));
+  HDDA_CUDA_TRY(scratch_alloc(&scratch, twopass_scratch_bytes(n), s));
   st = run_twopass(ro, rd, n, grid, lat, params->image_width, offsets, ray_idx, t0, t1,
                    capacity, &unused_total, scratch, nullptr, dev_status, s);
   cudaError_t e = cudaFreeAsync(scratch, s);

@@ -113,3 +113,51 @@ def test_async_argument_errors(H, frame):
     H.traverse_async(empty, empty, g, prm, e, st)
     torch.cuda.synchronize()
     assert int(e.offsets[0].item()) == 0 and int(st.item()) == 0
+
+
+def test_scratch_pool_streams_threads_and_capture(H):
+    """The calls' scratch comes from one pool per device: calls of different sizes on several
+    threads and streams, with synchronisations between, and a call captured into a CUDA graph
+    keep giving what one call alone gives."""
+    import threading
+    sc = scenes.tiny_scene()
+    o, d = scenes.tiny_camera().rays()
+    p = sc.params
+    prm = H.make_params(p.near, p.far, p.step, p.cone, p.max_step, p.max_steps)
+    g = H.build_vdb(torch.from_numpy(sc.occ).cuda(), sc.aabbs)
+    sizes = [o.shape[0], 1000, 33]
+    rays = [(torch.from_numpy(o[:n]).cuda(), torch.from_numpy(d[:n]).cuda()) for n in sizes]
+    want = [tuple(t.clone() for t in H.traverse_hdda(a, b, g, prm).trimmed()) for a, b in rays]
+    bad = []
+
+    def work(i):
+        s = torch.cuda.Stream()
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        for j in range(20):
+            k = (i + j) % len(sizes)
+            out = H.alloc_samples(sizes[k], want[k][1].numel())
+            s.wait_stream(torch.cuda.current_stream())
+            H.traverse_async(*rays[k], g, prm, out, st, stream=s)
+            s.synchronize()
+            if not all(torch.equal(x, y) for x, y in zip(
+                    (out.offsets, out.ray_idx, out.t0, out.t1), want[k])):
+                bad.append((i, j))
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+    out = H.alloc_samples(sizes[0], want[0][1].numel())
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        H.traverse_async(*rays[0], g, prm, out, st, stream=s)
+    for _ in range(2):
+        out.t0.fill_(-1.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out.t0, want[0][2]) and torch.equal(out.offsets, want[0][0])

@@ -48,7 +48,7 @@ L2_FLUSH_BYTES = 256 << 20
 # evaluations it does make when its work counters are on ("composite_blob_evals"), which
 # the bench does in a separate untimed pass.
 COMPOSITE_FP32_PER_BLOB = 6
-KERNELS_PER_TIMER = {"build_vdb": 5}   # the builder's timer spans five kernels
+KERNELS_PER_TIMER = {"build_vdb": 4}   # the builder's timer spans four kernels
 # L2 hit rate and warp execution efficiency (active lanes per warp instruction) per kernel
 # from the ncu --set full captures (object frame, camera 0; unbounded: its first 200 image
 # rows); dropped like the traffic when a kernel changes.

@@ -6,20 +6,19 @@
 //   thresholds_kernel   exact per-axis voxel boundaries X[a] (one thread per
 //                       boundary, binary search over binary32 keys)
 //   pack_dense_kernel   uint8 voxels -> uint32 bit words, one ballot per word
-//   vdb_blocks_kernel   one warp per 8^3 block: 16 ballots give the 512-bit
-//                       leaf mask and the block's empty/partial/full state
+//   vdb_blocks_kernel   one warp per four 8^3 blocks in a z row (8 lanes each):
+//                       the 512-bit leaf masks and the blocks'
+//                       empty/partial/full states
 //   vdb_nodes_kernel    one 128-thread CTA per 16^3-block node: ballots over
 //                       the block states give the child and tile masks, a
 //                       CTA scan gives each mask word's leaf-count prefix
 //   vdb_finalize_kernel one CTA: scan of leaf counts over all nodes, global
 //                       leaf prefix per mask word, leaf and tile totals
-//   vdb_scatter_kernel  16 threads per partial block copy its mask into the
-//                       compact leaf pool
-//   region_map_kernel   one thread per 2^3-voxel cell: the refined tree's
-//                       region holding the cell, flattened into 16 bits (an
-//                       update that changes no block's state recomputes only
-//                       the changed blocks' cells: region_map_blocks_kernel)
-// The node and scatter kernels also write the refinement masks (occupied
+//   vdb_finish_kernel   one warp per four blocks again: partial blocks' masks
+//                       into the compact leaf pool with their refinement
+//                       masks, and the region map of every block (an update
+//                       that changes no block's state: of the changed blocks)
+// The node and finish kernels also write the refinement masks (occupied
 // 32^3 and 16^3 groups per node, occupied 4^3 and 2^3 cells per leaf) that
 // let hierarchical DDA cross empty space in power-of-two steps below and
 // above the 8^3 leaf, in the manner of an octree (Sec. 5 suggests finer
@@ -101,47 +100,128 @@ __global__ void pack_dense_kernel(const uint8_t* __restrict__ dense, int L, int 
   if (w0 + lane < total) bits[w0 + lane] = mine;
 }
 
-// The 512 occupancy bits of the 8^3 block (bx, by, bz) of one level, voxel
-// ((x%8)*8 + y%8)*8 + z%8 at bit v%32 of word v/32: lane w < 16 receives word
-// w.  Every lane loads its 16 voxels first, so the loads are in flight
-// together, then the warp votes word by word.  Voxels past the grid's edge
-// are empty.
-__device__ __forceinline__ uint32_t block_words(const uint8_t* __restrict__ lvl, int R, int bx,
-                                                int by, int bz, int lane) {
-  uint32_t mine = 0;
-  // the 16 voxels of each lane first (loads in flight together), then the votes
-  uint8_t on[16];
-#pragma unroll
-  for (int w = 0; w < 16; ++w) {
-    const int v = w * 32 + lane;  // local voxel ((x%8)*8 + y%8)*8 + z%8
-    const int x = bx * 8 + (v >> 6), y = by * 8 + ((v >> 3) & 7), z = bz * 8 + (v & 7);
-    on[w] = 0;
-    if (x < R && y < R && z < R) on[w] = __ldg(lvl + ((int64_t)x * R + y) * R + z);
-  }
-#pragma unroll
-  for (int w = 0; w < 16; ++w) {
-    const uint32_t bal = __ballot_sync(kFull, on[w] != 0);
-    if (lane == w) mine = bal;
-  }
-  return mine;
+// Work on blocks is laid out four blocks per warp, eight lanes per block: lane
+// 4 y + j is lane y of slot j, so that the rows of four blocks side by side in z
+// make whole 32-byte sectors.
+struct BlockAt {
+  int l, bx, by, bz;
+};
+
+__device__ __forceinline__ BlockAt block_at(uint32_t blk, int B) {  // L * B^3 <= 8 * 128^3
+  BlockAt a;
+  a.bz = (int)(blk % (uint32_t)B);
+  blk /= (uint32_t)B;
+  a.by = (int)(blk % (uint32_t)B);
+  blk /= (uint32_t)B;
+  a.bx = (int)(blk % (uint32_t)B);
+  a.l = (int)(blk / (uint32_t)B);
+  return a;
 }
 
-__global__ void vdb_blocks_kernel(const uint8_t* __restrict__ dense, int L, int R, int B,
-                                  uint32_t* __restrict__ blk_masks,
-                                  uint8_t* __restrict__ blk_state) {
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t B3 = (int64_t)B * B * B;
-  if (warp >= (int64_t)L * B3) return;  // uniform per warp
-  const int l = (int)(warp / B3);
-  const int64_t b = warp % B3;
-  const int bx = (int)(b / ((int64_t)B * B)), by = (int)((b / B) % B), bz = (int)(b % B);
-  const uint8_t* lvl = dense + (int64_t)l * R * R * R;
-  const uint32_t mine = block_words(lvl, R, bx, by, bz, lane);
-  const bool any = __any_sync(kFull, lane < 16 && mine != 0u);
-  const bool all = __all_sync(kFull, lane >= 16 || mine == kFull);
-  if (lane < 16) blk_masks[warp * 16 + lane] = mine;
-  if (lane == 0) blk_state[warp] = all ? kBlockFull : (any ? kBlockPartial : kBlockEmpty);
+// Bit b of the result: byte b of the two words is not zero.
+__device__ __forceinline__ uint32_t nonzero8(uint2 v) {
+  const uint32_t f = ((((v.x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.x) >> 7) & 0x01010101u;
+  const uint32_t h = ((((v.y & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.y) >> 7) & 0x01010101u;
+  return __dp4a(h, 0x80402010u, __dp4a(f, 0x08040201u, 0u));
+}
+
+// The 512 occupancy bits of the lane's block, voxel ((x%8)*8 + y%8)*8 + z%8 at
+// bit v%32 of word v/32: lane y of the slot returns words 2 y and 2 y + 1,
+// the eight z rows of x = y, one byte per row.  The lane loads the rows of its
+// own y (all eight in flight together; kVec: R a multiple of 8, eight bytes
+// at once), and an 8 x 8 byte transpose over the slot's lanes turns (y, x) into
+// (x, y).  Voxels past the grid's edge are empty.
+template <bool kVec>
+__device__ __forceinline__ uint2 block_words(const uint8_t* __restrict__ dense, int R,
+                                             const BlockAt& a, bool active) {
+  const int lane = threadIdx.x & 31, y = lane >> 2;
+  uint32_t lo = 0, hi = 0;  // bytes x = 0..3 and 4..7 of this y
+  const int vy = a.by * 8 + y, vz = a.bz * 8;
+  const uint8_t* row = dense + (((int64_t)a.l * R + a.bx * 8) * R + vy) * R + vz;
+  if constexpr (kVec) {
+    uint2 v[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+      v[x] = active ? __ldg(reinterpret_cast<const uint2*>(row + (int64_t)x * R * R))
+                    : make_uint2(0u, 0u);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      lo |= nonzero8(v[x]) << (8 * x);
+      hi |= nonzero8(v[x + 4]) << (8 * x);
+    }
+  } else {
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      uint32_t b = 0;
+      if (active && vy < R && a.bx * 8 + x < R) {
+#pragma unroll
+        for (int z = 0; z < 8; ++z)
+          if (vz + z < R) b |= (__ldg(row + (int64_t)x * R * R + z) != 0 ? 1u : 0u) << z;
+      }
+      if (x < 4) lo |= b << (8 * x);
+      else hi |= b << (8 * (x - 4));
+    }
+  }
+  // transpose: halves of x against y ^ 4, then pairs against y ^ 2, then bytes against y ^ 1
+  const bool u4 = y & 4, u2 = y & 2, u1 = y & 1;
+  const uint32_t r4 = __shfl_xor_sync(kFull, u4 ? lo : hi, 16);
+  const uint32_t A = u4 ? r4 : lo, Bq = u4 ? hi : r4;  // rows y & 3 and (y & 3) + 4
+  const uint32_t k2 = __byte_perm(A, Bq, u2 ? 0x7632 : 0x5410);
+  const uint32_t r2 = __shfl_xor_sync(kFull, __byte_perm(A, Bq, u2 ? 0x5410 : 0x7632), 8);
+  const uint32_t own = __byte_perm(k2, r2, u1 ? 0x7531 : 0x6420);  // rows y, y+4, y^2, (y^2)+4
+  const uint32_t r1 = __shfl_xor_sync(kFull, __byte_perm(k2, r2, u1 ? 0x6420 : 0x7531), 4);
+  const uint32_t order = (y & 3) == 0 ? 0x3120u : (y & 3) == 1 ? 0x1302u
+                         : (y & 3) == 2 ? 0x2031u : 0x0213u;
+  return make_uint2(__byte_perm(__byte_perm(own, r1, 0x6420), 0u, order),
+                    __byte_perm(__byte_perm(own, r1, 0x7531), 0u, order));
+}
+
+// The slot's lanes, and its block's state from the lanes' words.
+__device__ __forceinline__ unsigned slot_lanes() { return 0x11111111u << (threadIdx.x & 3); }
+
+__device__ __forceinline__ uint8_t block_state(uint2 w) {
+  const unsigned m = slot_lanes();
+  const bool any = (__ballot_sync(kFull, (w.x | w.y) != 0u) & m) != 0u;
+  const bool all = (__ballot_sync(kFull, (w.x & w.y) == kFull) & m) == m;
+  return all ? kBlockFull : any ? kBlockPartial : kBlockEmpty;
+}
+
+// The block of the lane's slot in the i-th group of four along z of a grid
+// of B^3 blocks per level; false past the row's end.
+__device__ __forceinline__ bool quad_block(uint32_t i, int B, BlockAt& a) {
+  const uint32_t Q = ((uint32_t)B + 3) / 4;
+  a.bz = (int)(i % Q) * 4 + (threadIdx.x & 3);
+  i /= Q;
+  a.by = (int)(i % (uint32_t)B);
+  i /= (uint32_t)B;
+  a.bx = (int)(i % (uint32_t)B);
+  a.l = (int)(i / (uint32_t)B);
+  return a.bz < B;
+}
+
+__device__ __forceinline__ uint32_t block_index(const BlockAt& a, int B) {
+  return (((uint32_t)a.l * B + a.bx) * B + a.by) * B + a.bz;
+}
+
+// Bound by the occupancy bytes' read and issue (2 x 512^3: 58 us, 72 % of cycles
+// issuing; reading the bytes at 6.8 TB/s takes 40).  Single-byte loads, a ballot
+// per 32 voxels and a warp per block were what it replaces.
+template <bool kVec>
+__global__ void __launch_bounds__(256) vdb_blocks_kernel(const uint8_t* __restrict__ dense,
+                                                         uint32_t quads, int R, int B,
+                                                         uint32_t* __restrict__ blk_masks,
+                                                         uint8_t* __restrict__ blk_state) {
+  const uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (q >= quads) return;  // uniform per warp
+  BlockAt a;
+  const bool active = quad_block(q, B, a);
+  const uint2 w = block_words<kVec>(dense, R, a, active);
+  const uint8_t st = block_state(w);
+  if (!active) return;
+  const uint32_t blk = block_index(a, B);
+  const int y = (threadIdx.x & 31) >> 2;
+  *reinterpret_cast<uint2*>(blk_masks + (size_t)blk * kLeafWords + 2 * y) = w;
+  if (y == 0) blk_state[blk] = st;
 }
 
 // Exclusive CTA-wide scan of one uint32 per thread (blockDim.x <= 1024, multiple of 32).
@@ -292,253 +372,184 @@ __global__ void vdb_finalize_kernel(int64_t nodes, const uint32_t* __restrict__ 
   }
 }
 
-// Copies the mask of partial block `blk` into its slot of the compact leaf
-// pool and writes the leaf's refinement masks (occupied 2^3 and 4^3 cells,
-// fully occupied 2^3 cells).  Called by the 16 threads of one aligned
-// half-warp, `part` = 0..15, all of them together.
-__device__ __forceinline__ void scatter_block(int64_t blk, int part, int B, int N,
-                                              const uint32_t* __restrict__ blk_masks,
-                                              const uint32_t* __restrict__ child,
-                                              const uint32_t* __restrict__ prefix,
-                                              uint32_t* __restrict__ leaves,
-                                              uint32_t* __restrict__ lsub) {
-  const int64_t B3 = (int64_t)B * B * B;
-  const int l = (int)(blk / B3);
-  const int64_t b = blk % B3;
-  const int bx = (int)(b / ((int64_t)B * B)), by = (int)((b / B) % B), bz = (int)(b % B);
-  const int node = ((bx >> 4) * N + (by >> 4)) * N + (bz >> 4);
-  const int64_t ng = (int64_t)l * N * N * N + node;
-  const int cell = ((bx & 15) * 16 + (by & 15)) * 16 + (bz & 15);
-  const int w = cell >> 5;
-  const uint32_t bit = 1u << (cell & 31);
-  const uint32_t leaf = prefix[ng * kNodeWords + w] + __popc(child[ng * kNodeWords + w] & (bit - 1u));
-  leaves[(int64_t)leaf * kLeafWords + part] = blk_masks[blk * kLeafWords + part];
-  // refinement masks: each of the 16 threads classifies 4 of the 64 2^3
-  // cells; OR-reductions over the aligned half-warp join them
-  const unsigned half = 0xFFFFu << (threadIdx.x & 16);
-  const uint32_t* m = blk_masks + blk * kLeafWords;
-  uint32_t c2 = 0, f2 = 0, c4 = 0;  // bits of this thread's word (part >> 3) of c2/f2
-  for (int q = 0; q < 4; ++q) {
-    const int cell = 4 * part + q;  // 2^3 cells, (cx*4 + cy)*4 + cz
-    const int cx = cell >> 4, cy = (cell >> 2) & 3, cz = cell & 3;
-    bool any = false, all = true;
-    for (int a = 0; a < 8; ++a) {
-      const int v = ((2 * cx + (a >> 2)) * 8 + (2 * cy + ((a >> 1) & 1))) * 8 + 2 * cz + (a & 1);
-      const bool on = (__ldg(m + (v >> 5)) >> (v & 31)) & 1u;
-      any |= on;
-      all &= on;
-    }
-    if (any) {
-      c2 |= 1u << (cell & 31);
-      c4 |= 1u << (((cx >> 1) * 2 + (cy >> 1)) * 2 + (cz >> 1));
-    }
-    if (all) f2 |= 1u << (cell & 31);
-  }
-  uint32_t c2w[2] = {part < 8 ? c2 : 0u, part < 8 ? 0u : c2};
-  uint32_t f2w[2] = {part < 8 ? f2 : 0u, part < 8 ? 0u : f2};
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
-    c2w[0] |= __shfl_xor_sync(half, c2w[0], o);
-    c2w[1] |= __shfl_xor_sync(half, c2w[1], o);
-    f2w[0] |= __shfl_xor_sync(half, f2w[0], o);
-    f2w[1] |= __shfl_xor_sync(half, f2w[1], o);
-    c4 |= __shfl_xor_sync(half, c4, o);
-  }
-  if (part == 0) {
-    uint32_t* out = lsub + (int64_t)leaf * kLeafSubWords;
-    out[0] = c2w[0];
-    out[1] = c2w[1];
-    out[2] = c4;
-    out[3] = f2w[0];
-    out[4] = f2w[1];
-  }
-}
-
-__global__ void vdb_scatter_kernel(int L, int B, int N, const uint8_t* __restrict__ blk_state,
-                                   const uint32_t* __restrict__ blk_masks,
-                                   const uint32_t* __restrict__ child,
-                                   const uint32_t* __restrict__ prefix,
-                                   uint32_t* __restrict__ leaves, uint32_t* __restrict__ lsub,
-                                   const unsigned* __restrict__ gate) {
-  if (gate && *gate == 0u) return;
-  // grid-stride, so that an update can launch a small grid that exits at once when
-  // gated off; the stride is a multiple of 16, so a half-warp stays on one block
-  const int64_t total = (int64_t)L * B * B * B * 16;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t blk = t >> 4;
-    if (blk_state[blk] != kBlockPartial) continue;
-    scatter_block(blk, (int)(t & 15), B, N, blk_masks, child, prefix, leaves, lsub);
-  }
-}
-
-// Incremental update, step 1: one warp per listed block (every block when
-// `list` is null).  The block's mask and state are recomputed from the dense
+// Incremental update, step 1: four listed blocks per warp (every block when
+// `list` is null).  A block's mask and state are recomputed from the dense
 // bytes; a mask that differs is stored and changed[i] set, and flags[0] is
 // set when the block's state (empty, partial, full) changes, since the node
 // masks and the leaf compaction then change too.  An index outside the grid
 // is skipped and raises kDevBadIndex.
-__global__ void vdb_update_blocks_kernel(const uint8_t* __restrict__ dense, int L, int R, int B,
-                                         const int64_t* __restrict__ list, int64_t count,
-                                         uint32_t* __restrict__ blk_masks,
-                                         uint8_t* __restrict__ blk_state,
-                                         uint8_t* __restrict__ changed, unsigned* __restrict__ flags,
-                                         unsigned* __restrict__ status) {
-  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (i >= count) return;  // uniform per warp
-  const int64_t B3 = (int64_t)B * B * B;
-  const int64_t blk = list ? list[i] : i;
-  if (blk < 0 || blk >= (int64_t)L * B3) {
-    if (lane == 0) {
-      changed[i] = 0;
-      atomicOr(status, kDevBadIndex);
-    }
-    return;
-  }
-  const int l = (int)(blk / B3);
-  const int64_t b = blk % B3;
-  const int bx = (int)(b / ((int64_t)B * B)), by = (int)((b / B) % B), bz = (int)(b % B);
-  const uint8_t* lvl = dense + (int64_t)l * R * R * R;
-  const uint32_t mine = block_words(lvl, R, bx, by, bz, lane);
-  const uint32_t old = lane < 16 ? blk_masks[blk * kLeafWords + lane] : 0u;
-  const bool diff = __any_sync(kFull, lane < 16 && mine != old);
-  const bool any = __any_sync(kFull, lane < 16 && mine != 0u);
-  const bool all = __all_sync(kFull, lane >= 16 || mine == kFull);
-  const uint8_t st = all ? kBlockFull : (any ? kBlockPartial : kBlockEmpty);
-  if (diff && lane < 16) blk_masks[blk * kLeafWords + lane] = mine;
-  if (lane == 0) {
+template <bool kVec>
+__global__ void __launch_bounds__(256) vdb_update_blocks_kernel(
+    const uint8_t* __restrict__ dense, int L, int R, int B, const int64_t* __restrict__ list,
+    int64_t count, uint32_t* __restrict__ blk_masks, uint8_t* __restrict__ blk_state,
+    uint8_t* __restrict__ changed, unsigned* __restrict__ flags, unsigned* __restrict__ status) {
+  const int64_t i0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 4;
+  if (i0 >= count) return;  // uniform per warp
+  const int lane = threadIdx.x & 31, y = lane >> 2;
+  const int64_t i = i0 + (lane & 3);
+  const int64_t blk = i < count ? (list ? list[i] : i) : -1;
+  const bool active = blk >= 0 && blk < (int64_t)L * B * B * B;
+  const BlockAt a = block_at(active ? (uint32_t)blk : 0u, B);
+  const uint2 w = block_words<kVec>(dense, R, a, active);
+  const uint8_t st = block_state(w);
+  uint2* mask = reinterpret_cast<uint2*>(blk_masks + (active ? blk : 0) * kLeafWords) + y;
+  const uint2 old = active ? *mask : w;
+  const bool diff =
+      (__ballot_sync(kFull, active && (w.x != old.x || w.y != old.y)) & slot_lanes()) != 0u;
+  if (active && diff) *mask = w;
+  if (y == 0 && i < count) {
     changed[i] = diff ? 1 : 0;
-    if (st != blk_state[blk]) {
+    if (!active) {
+      atomicOr(status, kDevBadIndex);
+    } else if (st != blk_state[blk]) {
       blk_state[blk] = st;
       flags[0] = 1u;
     }
   }
 }
 
-// Incremental update, last step when no block changed state: the changed
-// partial blocks' leaves are rewritten in place (16 threads per listed
-// block); the tree's structure and every other leaf stay as they are.
-__global__ void vdb_rewrite_leaves_kernel(int B, int N, const int64_t* __restrict__ list,
-                                          int64_t count, const uint8_t* __restrict__ changed,
-                                          const unsigned* __restrict__ flags,
-                                          const uint8_t* __restrict__ blk_state,
-                                          const uint32_t* __restrict__ blk_masks,
-                                          const uint32_t* __restrict__ child,
-                                          const uint32_t* __restrict__ prefix,
-                                          uint32_t* __restrict__ leaves,
-                                          uint32_t* __restrict__ lsub) {
-  if (*flags != 0u) return;  // the structure changed: the full scatter ran instead
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = t >> 4;
-  if (i >= count || !changed[i]) return;
-  const int64_t blk = list ? list[i] : i;
-  if (blk_state[blk] != kBlockPartial) return;
-  scatter_block(blk, (int)(t & 15), B, N, blk_masks, child, prefix, leaves, lsub);
+// A pattern of bits 0, 2, 4, 6 as a nibble.
+__device__ __forceinline__ uint32_t nibble(uint32_t v) {
+  v = (v | (v >> 1)) & 0x33u;
+  return (v | (v >> 2)) & 0xfu;
+}
+
+// ORs a value over the lanes of each slot.
+__device__ __forceinline__ uint32_t slot_or(uint32_t v) {
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) v |= __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+// The last step of a build or update, four blocks per warp: a partial block's
+// mask goes into its slot of the compact leaf pool with the leaf's refinement
+// masks (occupied 2^3 and 4^3 cells, fully occupied 2^3 cells), and the
+// block's 4^3 region-map cells are written (layout in hdda_internal.cuh).
+// Lane y of a slot takes the cell rows y and y + 8, row = cx * 4 + cy: four
+// cells along z, one 8-byte store (kVec: R a multiple of 8).  A block that is
+// not partial has one region throughout, read from its node; a partial
+// block's cells follow from the bytes of four voxel rows, its 4^3 cells from
+// the rows' neighbours (lanes y ^ 1 and y ^ 4).  Voxels past the grid edge are
+// empty in the masks.
+//
+// `flags` null: every block.  Otherwise an update: every block if flags[0]
+// says that some block changed its state, and only the listed blocks with
+// changed[i] set if not.  Grid-stride, so that an update can launch one
+// resident wave.  Bound by the map's write (2 bytes per 2^3 voxels) and issue.
+// For 2 x 512^3 voxels this takes 43 us; with a thread per cell that descended the
+// tree and a scatter of 16 threads per block before it, the whole rebuild took
+// 499 us where it takes 113 now (1 x 128^3: 27.5 -> 21, 4 x 128^3: 42.6 -> 23; an
+// in-place update of 1 % of the blocks 264 -> 67, 40 -> 24 and 52 -> 25).
+template <bool kVec>
+__global__ void __launch_bounds__(256) vdb_finish_kernel(
+    GridDev g, uint32_t quads, const uint8_t* __restrict__ blk_state,
+    const uint32_t* __restrict__ blk_masks, uint32_t* __restrict__ leaves,
+    uint32_t* __restrict__ lsub, uint16_t* __restrict__ rmap, const unsigned* __restrict__ flags,
+    const int64_t* __restrict__ list, int64_t count, const uint8_t* __restrict__ changed) {
+  const bool all = !flags || *flags != 0u;
+  const int64_t items = all ? (int64_t)quads : (count + 3) / 4;
+  const int lane = threadIdx.x & 31, y = lane >> 2;
+  const int B = g.B, N = g.N, C = (g.R + 1) >> 1;
+  const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t it = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; it < items;
+       it += stride) {  // uniform per warp
+    BlockAt a;
+    bool active;
+    if (all) {
+      active = quad_block((uint32_t)it, B, a);
+    } else {
+      const int64_t i = it * 4 + (lane & 3);
+      active = i < count && changed[i];
+      a = block_at(active ? (uint32_t)(list ? list[i] : i) : 0u, B);
+    }
+    const uint32_t blk = active ? block_index(a, B) : 0u;
+    const uint8_t st = active ? blk_state[blk] : kBlockEmpty;
+    const int ng = ((a.l * N + (a.bx >> 4)) * N + (a.by >> 4)) * N + (a.bz >> 4);
+    const bool part = active && st == kBlockPartial;
+    uint32_t one = 0;  // the entry of a block with one region
+    if (active && !part) {
+      const uint32_t ns = g.nstate[ng];
+      if (ns != kNodeMixed) {
+        one = (kMapNodeLog2 << 8) | (ns == kNodeFull ? 0xffu : 0u);
+      } else if (st == kBlockFull) {
+        one = (3u << 8) | 0xffu;
+      } else {
+        const uint32_t* sup = g.nsuper + ng * kSuperWords;
+        const int g4 = (((a.bx >> 2) & 3) * 4 + ((a.by >> 2) & 3)) * 4 + ((a.bz >> 2) & 3);
+        const int g2 = (((a.bx >> 1) & 7) * 8 + ((a.by >> 1) & 7)) * 8 + ((a.bz >> 1) & 7);
+        one = !((sup[g4 >> 5] >> (g4 & 31)) & 1u)         ? 5u << 8
+              : !((sup[2 + (g2 >> 5)] >> (g2 & 31)) & 1u) ? 4u << 8
+                                                          : 3u << 8;
+      }
+    }
+    uint2 cells[2];  // four 16-bit entries of the rows y and y + 8
+    cells[0] = cells[1] = make_uint2(one | (one << 16), one | (one << 16));
+    if (__any_sync(kFull, part)) {  // uniform
+      const uint8_t* bytes = reinterpret_cast<const uint8_t*>(blk_masks + (size_t)blk * kLeafWords);
+      uint32_t c2[2], f2[2], c4 = 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int cx = 2 * h + (y >> 2), cy = y & 3;
+        uint32_t v0 = 0, v1 = 0;  // rows (2 cx, 2 cy), (2 cx, 2 cy + 1); the same of 2 cx + 1
+        if (part) {
+          v0 = *reinterpret_cast<const uint16_t*>(bytes + 16 * cx + 2 * cy);
+          v1 = *reinterpret_cast<const uint16_t*>(bytes + 16 * cx + 8 + 2 * cy);
+        }
+        const uint32_t p0 = v0 & 0xffu, p1 = v0 >> 8, p2 = v1 & 0xffu, p3 = v1 >> 8;
+        const uint32_t o = p0 | p1 | p2 | p3, n = p0 & p1 & p2 & p3;
+        const uint32_t any = (o | (o >> 1)) & 0x55u, full = n & (n >> 1) & 0x55u;
+        // over the 4^3 cells: some voxel (low half), some voxel missing (high half)
+        uint32_t c = any | ((~full & 0x55u) << 16);
+        c |= __shfl_xor_sync(kFull, c, 4);
+        c |= __shfl_xor_sync(kFull, c, 16);
+        uint32_t e[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const uint32_t m = ((p0 >> (2 * z)) & 3u) | (((p1 >> (2 * z)) & 3u) << 2) |
+                             (((p2 >> (2 * z)) & 3u) << 4) | (((p3 >> (2 * z)) & 3u) << 6);
+          const uint32_t big = c >> (4 * (z >> 1));
+          e[z] = !(big & 0x5u)            ? 2u << 8
+                 : !((big >> 16) & 0x5u)  ? (2u << 8) | 0xffu
+                 : m == 0u || m == 0xffu  ? (1u << 8) | m
+                                          : m;
+        }
+        if (part) cells[h] = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+        // the leaf's masks: cell (cx * 4 + cy) * 4 + cz, 4^3 cell ((cx/2) * 2 + cy/2) * 2 + cz/2
+        c2[h] = slot_or(nibble(any) << (4 * y));
+        f2[h] = slot_or(nibble(full) << (4 * y));
+        c4 |= (((c & 0x5u) ? 1u : 0u) | ((c & 0x50u) ? 2u : 0u)) << (4 * h + 2 * (cy >> 1));
+      }
+      c4 = slot_or(c4);
+      if (part) {
+        const int cell = ((a.bx & 15) * 16 + (a.by & 15)) * 16 + (a.bz & 15);
+        const int w = ng * kNodeWords + (cell >> 5);
+        const uint32_t leaf = g.prefix[w] + __popc(g.child[w] & ((1u << (cell & 31)) - 1u));
+        reinterpret_cast<uint2*>(leaves + (size_t)leaf * kLeafWords)[y] =
+            reinterpret_cast<const uint2*>(bytes)[y];
+        uint32_t* sub = lsub + (size_t)leaf * kLeafSubWords;
+        if (y < kLeafSubWords)
+          sub[y] = y == 0 ? c2[0] : y == 1 ? c2[1] : y == 2 ? c4 : y == 3 ? f2[0] : f2[1];
+      }
+    }
+    if (!active) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int cx = 4 * a.bx + 2 * h + (y >> 2), cy = 4 * a.by + (y & 3), cz = 4 * a.bz;
+      uint16_t* out = rmap + (((int64_t)a.l * C + cx) * C + cy) * C + cz;
+      if constexpr (kVec) {
+        *reinterpret_cast<uint2*>(out) = cells[h];
+      } else if (cx < C && cy < C) {  // past the grid edge when R is no multiple of 8
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+          if (cz + z < C)
+            out[z] = (uint16_t)((z < 2 ? cells[h].x : cells[h].y) >> (16 * (z & 1)));
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
 // host side
-// The region map (layout in hdda_internal.cuh), written after the tree and
-// its refinement masks.  Each thread descends the refined tree from the
-// cell's first voxel, exactly as a walk over the tree would: node state,
-// empty 32^3 and 16^3 groups, empty or tiled 8^3 block, empty or full 4^3
-// cell (full: its eight 2^3 cells are), empty or full 2^3 cell; a cell that
-// is none of these keeps its 8 voxel bits.  Voxels past the grid edge (odd R) are empty in the leaves.
-__device__ __forceinline__ uint16_t region_map_cell(const GridDev& g, int64_t idx) {
-  const int C = (g.R + 1) >> 1;
-  int64_t q = idx;
-  const int a2 = (int)(q % C);
-  q /= C;
-  const int a1 = (int)(q % C);
-  q /= C;
-  const int a0 = (int)(q % C);
-  const int l = (int)(q / C);
-  const int i[3] = {2 * a0, 2 * a1, 2 * a2};
-  const int N = g.N;
-  const int ng = l * N * N * N + ((i[0] >> 7) * N + (i[1] >> 7)) * N + (i[2] >> 7);
-  uint32_t lg = 0, mask = 0;
-  do {
-    const uint32_t st = g.nstate[ng];
-    if (st != kNodeMixed) {
-      lg = kMapNodeLog2;
-      mask = st == kNodeFull ? 0xffu : 0u;
-      break;
-    }
-    const uint32_t* ns = g.nsuper + ng * kSuperWords;
-    const int g4 = (((i[0] >> 5) & 3) * 4 + ((i[1] >> 5) & 3)) * 4 + ((i[2] >> 5) & 3);
-    if (!((ns[g4 >> 5] >> (g4 & 31)) & 1u)) { lg = 5; break; }
-    const int g2 = (((i[0] >> 4) & 7) * 8 + ((i[1] >> 4) & 7)) * 8 + ((i[2] >> 4) & 7);
-    if (!((ns[2 + (g2 >> 5)] >> (g2 & 31)) & 1u)) { lg = 4; break; }
-    const int cell = (((i[0] >> 3) & 15) * 16 + ((i[1] >> 3) & 15)) * 16 + ((i[2] >> 3) & 15);
-    const int w = cell >> 5;
-    const uint32_t bit = 1u << (cell & 31);
-    const uint32_t cw = g.child[ng * kNodeWords + w];
-    if (!(cw & bit)) {
-      lg = 3;
-      mask = (g.tile[ng * kNodeWords + w] & bit) ? 0xffu : 0u;
-      break;
-    }
-    const uint32_t leaf = g.prefix[ng * kNodeWords + w] + __popc(cw & (bit - 1u));
-    const uint32_t* ls = g.lsub + leaf * (uint32_t)kLeafSubWords;
-    const int c4 = (((i[0] >> 2) & 1) * 2 + ((i[1] >> 2) & 1)) * 2 + ((i[2] >> 2) & 1);
-    if (!((ls[2] >> c4) & 1u)) { lg = 2; break; }
-    // a 4^3 cell is full when its eight 2^3 cells are: bits base + {0, 1, 4, 5, 16, 17,
-    // 20, 21} of the leaf's 64-bit full-cell mask
-    const uint64_t full2 = (uint64_t)ls[3] | ((uint64_t)ls[4] << 32);
-    const int base4 = 32 * ((i[0] >> 2) & 1) + 8 * ((i[1] >> 2) & 1) + 2 * ((i[2] >> 2) & 1);
-    if (((full2 >> base4) & 0x330033ull) == 0x330033ull) { lg = 2; mask = 0xffu; break; }
-    const int c2 = (((i[0] >> 1) & 3) * 4 + ((i[1] >> 1) & 3)) * 4 + ((i[2] >> 1) & 3);
-    lg = 1;
-    if (!((ls[c2 >> 5] >> (c2 & 31)) & 1u)) break;          // empty 2^3 cell
-    if ((ls[3 + (c2 >> 5)] >> (c2 & 31)) & 1u) { mask = 0xffu; break; }  // full 2^3 cell
-    lg = 0;
-    const uint32_t* lw = g.leaves + leaf * (uint32_t)kLeafWords;
-    for (int u = 0; u < 8; ++u) {
-      const int x = (i[0] & 7) + (u >> 2), y = (i[1] & 7) + ((u >> 1) & 1), z = (i[2] & 7) + (u & 1);
-      const int v = (x * 8 + y) * 8 + z;
-      mask |= ((lw[v >> 5] >> (v & 31)) & 1u) << u;
-    }
-  } while (false);
-  return (uint16_t)((lg << 8) | mask);
-}
-
-// The whole map, one thread per cell.  With `flags` (an update), only when
-// the update changed the tree's structure.
-__global__ void region_map_kernel(GridDev g, uint16_t* __restrict__ rmap,
-                                  const unsigned* __restrict__ flags) {
-  if (flags && *flags == 0u) return;
-  const int C = (g.R + 1) >> 1;
-  const int64_t cells = (int64_t)g.L * C * C * C;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < cells;
-       idx += (int64_t)gridDim.x * blockDim.x)  // grid-stride, as vdb_scatter_kernel
-    rmap[idx] = region_map_cell(g, idx);
-}
-
-// An update that left every block's state as it was (so every node, group
-// and block region stays the same) changes the map only inside the blocks
-// whose voxels changed: their 4^3 cells are recomputed, 64 threads per block.
-__global__ void region_map_blocks_kernel(GridDev g, uint16_t* __restrict__ rmap,
-                                         const int64_t* __restrict__ list, int64_t count,
-                                         const uint8_t* __restrict__ changed,
-                                         const unsigned* __restrict__ flags) {
-  if (*flags != 0u) return;  // the structure changed: the whole map is recomputed
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = t >> 6;
-  if (i >= count || !changed[i]) return;
-  const int64_t blk = list ? list[i] : i;
-  const int B = g.B, C = (g.R + 1) >> 1;
-  const int64_t B3 = (int64_t)B * B * B;
-  const int l = (int)(blk / B3);
-  const int64_t b = blk % B3;
-  const int bx = (int)(b / ((int64_t)B * B)), by = (int)((b / B) % B), bz = (int)(b % B);
-  const int c = (int)(t & 63);
-  const int cx = 4 * bx + (c >> 4), cy = 4 * by + ((c >> 2) & 3), cz = 4 * bz + (c & 3);
-  if (cx >= C || cy >= C || cz >= C) return;  // past the grid edge (R not a multiple of 8)
-  const int64_t idx = (((int64_t)l * C + cx) * C + cy) * C + cz;
-  rmap[idx] = region_map_cell(g, idx);
-}
-
 // ---------------------------------------------------------------------------
 
 int validate(const uint8_t* dense, int levels, int res, const hdda_aabb* aabbs) {
@@ -600,9 +611,19 @@ size_t layout(hdda_grid* g, char* base) {
 
 unsigned blocks_for(int64_t threads, int per) { return (unsigned)((threads + per - 1) / per); }
 
-// CTAs of the update's gated grid-stride kernels: eight 256-thread CTAs per SM of a
-// 152-SM GB300, about one resident wave
+// CTAs of the update's grid-stride kernel: eight 256-thread CTAs per SM of a 152-SM GB300,
+// about one resident wave
 constexpr unsigned kGatedCtas = 152 * 8;
+
+// Groups of four blocks along z, and whether their voxel rows can be loaded
+// eight bytes at a time.
+uint32_t quad_count(const hdda_grid* g) {
+  return (uint32_t)((int64_t)g->L * g->B * g->B * ((g->B + 3) / 4));
+}
+
+bool vec_rows(const hdda_grid* g, const uint8_t* dense) {
+  return g->R % 8 == 0 && reinterpret_cast<uintptr_t>(dense) % 8 == 0;
+}
 
 int launch_build(hdda_grid* g, const uint8_t* dense, cudaStream_t s) {
   if (g->kind == HDDA_GRID_DENSE) {
@@ -612,10 +633,12 @@ int launch_build(hdda_grid* g, const uint8_t* dense, cudaStream_t s) {
     kt.stop();
     HDDA_CUDA_TRY(cudaGetLastError());
   } else {
-    const int64_t nblk = g->blocks_total();
-    KernelTimer kt("build_vdb", s);  // the five build kernels together
-    vdb_blocks_kernel<<<blocks_for(nblk * 32, 256), 256, 0, s>>>(dense, g->L, g->R, g->B,
-                                                                 g->blk_masks, g->blk_state);
+    KernelTimer kt("build_vdb", s);  // the four build kernels together
+    const uint32_t quads = quad_count(g);
+    const unsigned ctas = blocks_for((int64_t)quads * 32, 256);
+    const bool vec = vec_rows(g, dense);
+    (vec ? vdb_blocks_kernel<true> : vdb_blocks_kernel<false>)<<<ctas, 256, 0, s>>>(
+        dense, quads, g->R, g->B, g->blk_masks, g->blk_state);
     HDDA_CUDA_TRY(cudaGetLastError());
     vdb_nodes_kernel<<<(unsigned)g->nodes_total(), kNodeWords, 0, s>>>(
         g->L, g->B, g->N, g->blk_state, g->child, g->tile, g->local_prefix, g->node_leaves,
@@ -624,12 +647,9 @@ int launch_build(hdda_grid* g, const uint8_t* dense, cudaStream_t s) {
     vdb_finalize_kernel<<<1, 1024, 0, s>>>(g->nodes_total(), g->node_leaves, g->node_tiles,
                                           g->local_prefix, g->prefix, g->totals, nullptr);
     HDDA_CUDA_TRY(cudaGetLastError());
-    vdb_scatter_kernel<<<blocks_for(nblk * 16, 256), 256, 0, s>>>(
-        g->L, g->B, g->N, g->blk_state, g->blk_masks, g->child, g->prefix, g->leaves, g->lsub,
-        nullptr);
-    HDDA_CUDA_TRY(cudaGetLastError());
-    region_map_kernel<<<blocks_for(g->map_cells(), 256), 256, 0, s>>>(g->view(), g->rmap,
-                                                                       nullptr);
+    (g->R % 8 == 0 ? vdb_finish_kernel<true> : vdb_finish_kernel<false>)<<<ctas, 256, 0, s>>>(
+        g->view(), quads, g->blk_state, g->blk_masks, g->leaves, g->lsub, g->rmap, nullptr, nullptr,
+        0, nullptr);
     kt.stop();
     HDDA_CUDA_TRY(cudaGetLastError());
   }
@@ -743,8 +763,10 @@ int update_vdb(hdda_grid* g, const uint8_t* dense, const int64_t* blocks, int64_
   cudaError_t e = cudaMemsetAsync(scratch, 0, 16, s);
   if (e != cudaSuccess) st = cuda_error(e, "cudaMemsetAsync");
   if (st == HDDA_OK) {
-    KernelTimer kt("update_vdb", s);  // the update's seven kernels together
-    vdb_update_blocks_kernel<<<blocks_for(count * 32, 256), 256, 0, s>>>(
+    KernelTimer kt("update_vdb", s);  // the update's four kernels together
+    const unsigned ctas = blocks_for((count + 3) / 4 * 32, 256);
+    (vec_rows(g, dense) ? vdb_update_blocks_kernel<true>
+                        : vdb_update_blocks_kernel<false>)<<<ctas, 256, 0, s>>>(
         dense, g->L, g->R, g->B, blocks, count, g->blk_masks, g->blk_state, changed, flags,
         status);
     vdb_nodes_kernel<<<(unsigned)g->nodes_total(), kNodeWords, 0, s>>>(
@@ -752,18 +774,12 @@ int update_vdb(hdda_grid* g, const uint8_t* dense, const int64_t* blocks, int64_
         g->node_tiles, g->nstate, g->nsuper, flags);
     vdb_finalize_kernel<<<1, 1024, 0, s>>>(g->nodes_total(), g->node_leaves, g->node_tiles,
                                           g->local_prefix, g->prefix, g->totals, flags);
-    // the gated kernels run as grid-stride loops over a grid of at most kGatedCtas CTAs,
-    // so that they cost next to nothing when the update changed no block's state
-    vdb_scatter_kernel<<<std::min(blocks_for(g->blocks_total() * 16, 256), kGatedCtas), 256, 0,
-                         s>>>(g->L, g->B, g->N, g->blk_state, g->blk_masks, g->child, g->prefix,
-                              g->leaves, g->lsub, flags);
-    vdb_rewrite_leaves_kernel<<<blocks_for(count * 16, 256), 256, 0, s>>>(
-        g->B, g->N, blocks, count, changed, flags, g->blk_state, g->blk_masks, g->child,
-        g->prefix, g->leaves, g->lsub);
-    region_map_kernel<<<std::min(blocks_for(g->map_cells(), 256), kGatedCtas), 256, 0, s>>>(
-        g->view(), g->rmap, flags);
-    region_map_blocks_kernel<<<blocks_for(count * 64, 256), 256, 0, s>>>(
-        g->view(), g->rmap, blocks, count, changed, flags);
+    // grid-stride over at most one resident wave: it costs little when no block changed state
+    const uint32_t quads = quad_count(g);
+    (g->R % 8 == 0 ? vdb_finish_kernel<true> : vdb_finish_kernel<false>)<<<
+        std::min(blocks_for((int64_t)quads * 32, 256), kGatedCtas), 256, 0, s>>>(
+        g->view(), quads, g->blk_state, g->blk_masks, g->leaves, g->lsub, g->rmap, flags, blocks,
+        count, changed);
     kt.stop();
     e = cudaGetLastError();
     if (e != cudaSuccess) st = cuda_error(e, "update kernels");

@@ -60,8 +60,8 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     const int64_t* __restrict__ offsets, const float* __restrict__ t0,
     const float* __restrict__ t1, const float* __restrict__ field, int G,
     float* __restrict__ rgba, bool count_evals) {
-  extern __shared__ __align__(16) unsigned char smem[];  // field_layout(G, kWarpsPerCta, R)
-  const FieldLayout L = field_layout(G, kWarpsPerCta, R);
+  extern __shared__ __align__(16) unsigned char smem[];  // field_layout
+  const FieldLayout L = field_layout(G, kWarpsPerCta, R, kMany ? 0 : kRing);
   stage_blobs(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, o, d, tb);
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, tb);
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
@@ -142,10 +142,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned)(min(q, end) - max(q - kChunk, beg));
-    shade_chunk(sums, dt, acc);
+    float2 f[kPairs];
+    shade_chunk(sums, dt, acc, f);
+    float* const keep = &fw.lens(L)[max(ray, 0)].x;  // free once the ray's records are set up
+    if constexpr (!kMany)
+      faint_chunk(reinterpret_cast<float*>(smem + fw.recs + L.ring), keep, f, ray, q - kChunk, beg,
+                  end, my_beg, acc.T);
     const bool done = ray >= 0 && q - kPerLane * gl >= end;
     if (__any_sync(kFieldFull, done)) {
-      finish_rays(acc, done, rgba + 4 * ray);
+      float T = acc.T;
+      if (!kMany && done && T > kFaint) T = *keep;
+      finish_rays(acc, T, done, rgba + 4 * ray);
       if (done) {
         ray = -1;
         beg = end = 0;
@@ -189,7 +196,7 @@ extern "C" int hdda_composite(const float* rays_o, const float* rays_d, int64_t 
   const int64_t blocks = (warps + kWarpsPerCta - 1) / kWarpsPerCta;
   if (blocks > INT32_MAX) return set_error(HDDA_ERR_INVALID_ARG, "too many rays");
   const unsigned grid = (unsigned)blocks;
-  const FieldLayout L = field_layout(n_gauss, kWarpsPerCta, R);
+  const FieldLayout L = field_layout(n_gauss, kWarpsPerCta, R, n_gauss <= kAllBlobs ? kRing : 0);
   const bool vec = ((reinterpret_cast<uintptr_t>(t0) | reinterpret_cast<uintptr_t>(t1)) & 15) == 0;
   const auto kern = n_gauss <= kAllBlobs
                         ? (vec ? composite_kernel<true, false> : composite_kernel<false, false>)

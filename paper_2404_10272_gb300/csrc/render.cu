@@ -17,8 +17,8 @@
 //
 // A ray with more than kMaxRuns runs is finished in rounds: after the runs
 // it has are composited, it walks again from the end of the last one
-// (walk_from) and the next kMaxRuns runs are composited with its optical
-// depth and colour carried over, so samples are still accumulated front to
+// (walk_from) and the next kMaxRuns runs are composited with its
+// transmittance and colour carried over, so samples are still accumulated front to
 // back.
 //
 // The same kernel with kStore also writes what the samplers' emit writes:
@@ -73,12 +73,12 @@ __device__ __forceinline__ int number_runs(uint2* sr, int nr) {
 template <int kMode, bool kStore, bool kMany>
 __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R, GridDev g,
-    LatticeDev lat, const uint8_t* __restrict__ nruns, const uint2* __restrict__ runs,
-    const float* __restrict__ field, int G, float* __restrict__ rgba, bool count_evals,
-    StoreArgs out) {
-  // field_layout(G, kRenderWarps, R), then [kRenderWarps][R][kRunStride] runs
+    LatticeDev lat, const uint8_t* __restrict__ nruns,
+    const uint2* __restrict__ runs, const float* __restrict__ field, int G,
+    float* __restrict__ rgba, bool count_evals, StoreArgs out) {
+  // field_layout, then [kRenderWarps][R][kRunStride] runs
   extern __shared__ __align__(16) unsigned char smem[];
-  const FieldLayout L = field_layout(G, kRenderWarps, R);
+  const FieldLayout L = field_layout(G, kRenderWarps, R, 0);
   stage_blobs(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, o, d, tb);
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, tb);
     my_w = number_runs(sr + lane * kRunStride, nr);
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned) min(kChunk, W - q);
-    shade_chunk(sums, dt, acc);
+    float2 f[kPairs];
+    shade_chunk(sums, dt, acc, f);
     q += kChunk;
     const bool round_over = ray >= 0 && q - kPerLane * gl >= W;
     bool done = round_over && k_next >= lat.K;
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
       }
     }
     if (__any_sync(kFull, done)) {
-      finish_rays(acc, done, rgba + 4 * ray);
+      finish_rays(acc, acc.T, done, rgba + 4 * ray);
       if (done) {
         ray = -1;
         W = 0;
@@ -287,15 +288,15 @@ int launch_field(const WalkArgs& w, const uint8_t* nr, const uint2* runs, const 
   const int R = field_task_rays(w.n);
   const int64_t warps = (w.n + R - 1) / R;
   const unsigned nb = (unsigned)((warps + kRenderWarps - 1) / kRenderWarps);
-  const size_t smem = field_layout(G, kRenderWarps, R).bytes +
+  const size_t smem = field_layout(G, kRenderWarps, R, 0).bytes +
                       (size_t)kRenderWarps * R * kRunStride * sizeof(uint2);
   const auto kern =
       G <= kAllBlobs ? render_kernel<kMode, kStore, false> : render_kernel<kMode, kStore, true>;
   if (smem > 48 * 1024)
     HDDA_CUDA_TRY(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<nb, kRenderWarps * 32, smem, s>>>(w.ro, w.rd, w.n, R, w.g, w.lat, nr, runs, field, G, rgba,
-                                           counters_on(), out);
+  kern<<<nb, kRenderWarps * 32, smem, s>>>(w.ro, w.rd, w.n, R, w.g, w.lat, nr, runs, field, G,
+                                           rgba, counters_on(), out);
   return HDDA_OK;
 }
 

@@ -6,14 +6,14 @@
 // own output buffers.  Every job's rays are cut into 32-ray tiles numbered
 // consecutively over all jobs.  batch_walk_kernel is persistent: each warp
 // takes `tiles_per_fetch` tiles at a time from one atomic counter (work
-// stealing), finds the job of each tile by binary search, copies that job's
-// grid descriptor into its own slice of shared memory when the job changes,
-// and walks the tile exactly as the single-call walk does.  One scan over all
-// tiles then gives every tile its offset; a job's offsets are those minus the
-// job's first prefix.  batch_emit_kernel writes each job's CSR offsets and
-// samples into that job's buffers, with the capacity checked per job.  With
-// these three kernels and a few memsets, a batch is one graph launch however
-// many jobs it holds; the sizes (block of the walk, tiles per fetch, warps per
+// stealing), finds a tile's job when it leaves the last one's tiles, copies the
+// job's descriptor into its own slice of shared memory then,
+// and walks the tile exactly as the single-call walk does, adding the tile's
+// samples to its job's group sums (tile_offset, walk.cuh).  batch_emit_kernel
+// finds each tile's offset within its job from those and writes the job's CSR
+// offsets and samples into the job's buffers, with the capacity checked per
+// job.  With these two kernels and a few memsets, a batch is one graph launch
+// however many jobs it holds; the sizes (block of the walk, tiles per fetch, warps per
 // emit CTA) are chosen by the autotuner in the Python package.
 #include <cstring>
 #include <new>
@@ -42,42 +42,57 @@ struct JobDev {
   int64_t tiles;
 };
 
+// The job's first entry among the batch's group sums of 2^shift tiles.  A
+// job's groups count from its own first tile, so its entries end before
+// group0 of the next job: floor(a) + ceil(b) <= floor(a + b) + 1.
+__host__ __device__ __forceinline__ int64_t group0(int64_t tile0, int j, int shift) {
+  return (tile0 >> shift) + j;
+}
+
 // Largest j with tile0[j] <= t (tile0 has J + 1 entries, tile0[J] = T).
+// Called by a whole warp with one t: each step reads up to 32 entries at once
+// and leaves the stretch between two of them, two dependent loads for up to
+// 1024 jobs where a binary search has ten.
 __device__ __forceinline__ int find_job(const int64_t* __restrict__ tile0, int J, int64_t t) {
-  int lo = 0, hi = J - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(tile0 + mid) <= t) lo = mid; else hi = mid - 1;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = J;  // the job is one of lo .. lo + n - 1, and tile0[lo] <= t
+  while (n > 1) {
+    const int step = (n + 31) >> 5, i = lane * step;
+    const unsigned le = __ballot_sync(kFull, i < n && __ldg(tile0 + lo + i) <= t);
+    const int k = (__popc(le) - 1) * step;  // tile0 does not decrease
+    lo += k;
+    n = min(step, n - k);
   }
   return lo;
 }
 
-constexpr int kGridWords = (sizeof(GridDev) + 3) / 4;
-
-// Copies a job's grid descriptor into a warp's shared-memory slot.
-__device__ __forceinline__ void warp_copy_grid(GridDev* dst, const GridDev* src) {
+// Copies a job's descriptor (or its grid's) into a warp's shared-memory slot.
+template <typename T>
+__device__ __forceinline__ void warp_copy(T* dst, const T* src) {
+  static_assert(sizeof(T) % 4 == 0, "copied by words");
   const uint32_t* s = reinterpret_cast<const uint32_t*>(src);
   uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  for (int i = threadIdx.x & 31; i < kGridWords; i += 32) d[i] = __ldg(s + i);
+  for (int i = threadIdx.x & 31; i < (int)(sizeof(T) / 4); i += 32) d[i] = __ldg(s + i);
   __syncwarp();
 }
 
+// Bounded by instruction issue (73 % of cycles issue, 22 of 32 lanes active).
+// What a job's rays share is read from shared memory as needed and the
+// registers are held to 64, so 32 warps fit an SM instead of 24: 64 cameras of
+// up to 800 x 800 pixels (12 M rays, 600 M samples) took 3960 us in all with 75
+// registers, 3877 with 64.
 template <int kMode, int kBlock, bool kSkip, bool kCheck>
-__global__ void __launch_bounds__(kBlock) batch_walk_kernel(
+__global__ void __launch_bounds__(kBlock, 1024 / kBlock) batch_walk_kernel(
     const JobDev* __restrict__ jobs, const int64_t* __restrict__ tile0, int J, int64_t T,
     int tiles_per_fetch, int32_t* __restrict__ counts, uint8_t* __restrict__ nruns_out,
-    uint2* __restrict__ runs, int64_t* __restrict__ tile_sum, unsigned* __restrict__ counter,
-    unsigned* __restrict__ status) {
-  __shared__ __align__(16) GridDev s_grid[kBlock / 32];
+    uint2* __restrict__ runs, int64_t* __restrict__ tile_sum,
+    unsigned long long* __restrict__ sums32, unsigned long long* __restrict__ sums1024,
+    unsigned* __restrict__ counter, unsigned* __restrict__ status) {
+  __shared__ __align__(16) JobDev s_job[kBlock / 32];  // the job in work, per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  GridDev& g = s_grid[warp];
+  JobDev& job = s_job[warp];
   const int64_t slots = T * 32;  // ray slots over the whole batch (stride of the runs)
   int cur = -1;
-  LatticeDev lat{};
-  LatHdr h{};
-  int64_t n = 0, job_tile0 = 0;
-  const float* ro = nullptr;
-  const float* rd = nullptr;
   for (;;) {
     unsigned first = 0;
     if (lane == 0) first = atomicAdd(counter, (unsigned)tiles_per_fetch);
@@ -85,57 +100,61 @@ __global__ void __launch_bounds__(kBlock) batch_walk_kernel(
     if ((int64_t)first >= T) break;
     const int64_t last = min((int64_t)first + tiles_per_fetch, T);
     for (int64_t t = first; t < last; ++t) {
-      const int j = find_job(tile0, J, t);
-      if (j != cur) {
-        cur = j;
-        warp_copy_grid(&g, &jobs[j].g);
-        lat = jobs[j].lat;
-        h = lat_hdr(lat);
-        n = jobs[j].n;
-        job_tile0 = jobs[j].tile0;
-        ro = jobs[j].ro;
-        rd = jobs[j].rd;
+      if (cur < 0 || t - job.tile0 >= job.tiles) {  // tiles come in order within a fetch
+        __syncwarp();  // every lane has read the old one
+        cur = find_job(tile0, J, t);
+        warp_copy(&job, jobs + cur);
       }
-      const int64_t lr = (t - job_tile0) * 32 + lane;
+      const int64_t lt = t - job.tile0, lr = lt * 32 + lane;
       const int64_t gr = t * 32 + lane;
       int64_t c = 0;
-      if (lr < n) {
+      if (lr < job.n) {
         Ray ray;
         int nr = 0;
-        if (load_ray(ro, rd, lr, ray))
-          c = walk<kMode, false, false, kSkip, kCheck>(g, global_tabs(g, lat), lat, h, ray, runs + gr,
-                                                       slots, nr, 0, 0, 0, nullptr, nullptr,
-                                                       nullptr, status);
+        if (load_ray(job.ro, job.rd, lr, ray))
+          c = walk<kMode, false, false, kSkip, kCheck>(
+              job.g, global_tabs(job.g, job.lat), job.lat, lat_hdr(job.lat), ray, runs + gr, slots,
+              nr, 0, 0, 0, nullptr, nullptr, nullptr, status);
         counts[gr] = (int32_t)c;
         nruns_out[gr] = (uint8_t)min(nr, 255);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-      if (lane == 0) tile_sum[t] = c;
+      if (lane == 0) {
+        tile_sum[t] = c;
+        atomicAdd(sums32 + group0(job.tile0, cur, 5) + (lt >> 5), (unsigned long long)c);
+        atomicAdd(sums1024 + group0(job.tile0, cur, 10) + (lt >> 10), (unsigned long long)c);
+      }
     }
   }
 }
 
+// Bounded by its stores (5.6 TB/s of 6.8 on that batch).  The chain in front of
+// them is kept short: the tile's counts are loaded beside the search for its
+// job, and the offset comes from three sets of sums read at once; a scan of
+// all tiles in a kernel of one CTA between the walk and this one took 100 of
+// 4240 us.  With 64 registers it spills (4010 instead of 3877 us).
 template <int kMode, int kWarps>
 __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
     const JobDev* __restrict__ jobs, const int64_t* __restrict__ tile0, int J, int64_t T,
     const int32_t* __restrict__ counts, const uint8_t* __restrict__ nruns,
-    const uint2* __restrict__ runs, const int64_t* __restrict__ tile_prefix,
-    const int64_t* __restrict__ grand_total, int64_t* __restrict__ job_totals,
+    const uint2* __restrict__ runs, const int64_t* __restrict__ tile_sum,
+    const unsigned long long* __restrict__ sums32,
+    const unsigned long long* __restrict__ sums1024, int64_t* __restrict__ job_totals,
     unsigned* __restrict__ job_status, unsigned* __restrict__ status) {
   __shared__ uint2 s_rec[kWarps][kRecMax + 1];
   __shared__ __align__(16) GridDev s_grid[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t t = (int64_t)blockIdx.x * kWarps + warp;
   if (t >= T) return;  // uniform per warp
+  const int64_t gr = t * 32 + lane;
+  int c = __ldg(counts + gr), nr = __ldg(nruns + gr);  // not written behind a job's rays
   const int j = find_job(tile0, J, t);
   const JobDev& jb = jobs[j];
   const int64_t jt0 = jb.tile0, n = jb.n, capacity = jb.capacity;
   const int64_t lr = (t - jt0) * 32 + lane;
-  const int64_t gr = t * 32 + lane;
   const int64_t slots = T * 32;
-  const int c = lr < n ? counts[gr] : 0;
-  const int nr = lr < n ? (int)nruns[gr] : 0;
+  if (lr >= n) c = nr = 0;
   // a tile holds at most 32 * 2^24 samples: 32-bit positions within it
   int inc = c;
 #pragma unroll
@@ -144,13 +163,13 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
     if (lane >= o) inc += y;
   }
   const int q = inc - c;
-  const int64_t base = __ldg(tile_prefix + jt0);
-  const int64_t wbeg = __ldg(tile_prefix + t) - base;  // the tile's first sample in the job
+  // the tile's first sample in the job
+  const int64_t wbeg = tile_offset(t - jt0, tile_sum + jt0, sums32 + group0(jt0, j, 5),
+                                   sums1024 + group0(jt0, j, 10));
   const int64_t off = wbeg + q;
   if (lr < n) jb.offsets[lr] = off;
-  if (t == jt0 + jb.tiles - 1 && lane == 0) {
-    const int64_t next = __ldg(tile0 + j + 1);
-    const int64_t total = (next < T ? __ldg(tile_prefix + next) : *grand_total) - base;
+  if (t == jt0 + jb.tiles - 1 && lane == 31) {
+    const int64_t total = wbeg + inc;
     jb.offsets[n] = total;
     job_totals[j] = total;
     if (capacity > 0 && total > capacity) atomicOr(job_status + j, kJobCapacity);
@@ -181,7 +200,7 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
   expand_records(rec, nrec, lim, wbeg, (int32_t)(lr - lane), lat.t, vec, jb.ray_idx, jb.t0,
                  jb.t1);
   if (__any_sync(kFull, overflow)) {
-    warp_copy_grid(&s_grid[warp], &jb.g);  // the whole warp copies; only overflowing lanes walk
+    warp_copy(&s_grid[warp], &jb.g);  // the whole warp copies; only overflowing lanes walk
     if (overflow) {
       Ray ray;
       load_ray(jb.ro, jb.rd, lr, ray);
@@ -217,9 +236,10 @@ struct hdda_batch {
   // carved from scratch
   unsigned* counter = nullptr;
   unsigned* status = nullptr;
-  int64_t* total = nullptr;
+  unsigned long long* sums32 = nullptr;  // group sums, behind the counter and the status
+  unsigned long long* sums1024 = nullptr;
+  size_t cleared = 0;                    // bytes from the counter to their end
   int64_t* tile_sum = nullptr;
-  int64_t* tile_prefix = nullptr;
   int32_t* counts = nullptr;
   uint8_t* nruns = nullptr;
   uint2* runs = nullptr;
@@ -266,7 +286,7 @@ void launch_batch_walk_c(const hdda_batch* b, cudaStream_t s) {
 #define HDDA_BATCH_WALK(BS)                                                              \
   batch_walk_kernel<kMode, BS, kSkip, kCheck><<<grid, BS, 0, s>>>(                       \
       b->jobs, b->tile0, b->n_jobs, b->T, tpf, b->counts, b->nruns, b->runs, b->tile_sum, \
-      b->counter, b->status)
+      b->sums32, b->sums1024, b->counter, b->status)
   switch (b->cfg.walk_block) {
     case 128: HDDA_BATCH_WALK(128); break;
     case 256: HDDA_BATCH_WALK(256); break;
@@ -291,8 +311,8 @@ template <int kMode>
 void launch_batch_emit(const hdda_batch* b, cudaStream_t s) {
 #define HDDA_BATCH_EMIT(W)                                                                    \
   batch_emit_kernel<kMode, W><<<(unsigned)((b->T + W - 1) / W), W * 32, 0, s>>>(             \
-      b->jobs, b->tile0, b->n_jobs, b->T, b->counts, b->nruns, b->runs, b->tile_prefix,      \
-      b->total, b->job_totals, b->job_status, b->status)
+      b->jobs, b->tile0, b->n_jobs, b->T, b->counts, b->nruns, b->runs, b->tile_sum,         \
+      b->sums32, b->sums1024, b->job_totals, b->job_status, b->status)
   switch (b->cfg.emit_warps) {
     case 2: HDDA_BATCH_EMIT(2); break;
     case 4: HDDA_BATCH_EMIT(4); break;
@@ -301,9 +321,9 @@ void launch_batch_emit(const hdda_batch* b, cudaStream_t s) {
 #undef HDDA_BATCH_EMIT
 }
 
-// Queues one execution of the batch on s (memsets, walk, scan, emit).
+// Queues one execution of the batch on s (memsets, walk, emit).
 int enqueue(const hdda_batch* b, cudaStream_t s) {
-  HDDA_CUDA_TRY(cudaMemsetAsync(b->scratch, 0, 256, s));
+  HDDA_CUDA_TRY(cudaMemsetAsync(b->scratch, 0, b->cleared, s));
   HDDA_CUDA_TRY(cudaMemsetAsync(b->job_totals, 0, sizeof(int64_t) * b->n_jobs, s));
   HDDA_CUDA_TRY(cudaMemsetAsync(b->job_status, 0, sizeof(unsigned) * b->n_jobs, s));
   for (int64_t* p : b->zero_offsets) HDDA_CUDA_TRY(cudaMemsetAsync(p, 0, sizeof(int64_t), s));
@@ -313,9 +333,6 @@ int enqueue(const hdda_batch* b, cudaStream_t s) {
     case kModeVdb: launch_batch_walk<kModeVdb>(b, s); break;
     default: launch_batch_walk<kModeVdbMap>(b, s); break;
   }
-  HDDA_CUDA_TRY(cudaGetLastError());
-  tile_scan_kernel<<<1, kScanThreads, 0, s>>>(b->tile_sum, b->T, b->tile_prefix, b->total,
-                                              b->total + 1);
   HDDA_CUDA_TRY(cudaGetLastError());
   switch (b->mode) {
     case kModeDense: launch_batch_emit<kModeDense>(b, s); break;
@@ -408,7 +425,9 @@ int create(const hdda_job* jobs, int n_jobs, const hdda_batch_config* cfg, hdda_
   b->cfg = c;
   b->zero_offsets = zero_offsets;
   const int64_t slots = T * 32;
-  b->scratch_bytes = 256 + 2 * a256(8 * (size_t)T + 8) + a256(4 * (size_t)slots) +
+  const size_t groups32 = (size_t)group0(T, n_jobs, 5), groups1024 = (size_t)group0(T, n_jobs, 10);
+  b->cleared = 256 + 8 * (groups32 + groups1024);
+  b->scratch_bytes = a256(b->cleared) + a256(8 * (size_t)T) + a256(4 * (size_t)slots) +
                      a256((size_t)slots) + a256(sizeof(uint2) * kMaxRuns * (size_t)slots) +
                      a256(8 * (size_t)n_jobs) + a256(4 * (size_t)n_jobs) +
                      a256(sizeof(JobDev) * n_jobs) + a256(8 * (size_t)(n_jobs + 1));
@@ -428,12 +447,11 @@ int create(const hdda_job* jobs, int n_jobs, const hdda_batch_config* cfg, hdda_
   char* p = b->scratch;
   b->counter = reinterpret_cast<unsigned*>(p);
   b->status = b->counter + 1;
-  b->total = reinterpret_cast<int64_t*>(p + 8);  // total and a spare word
-  p += 256;
+  b->sums32 = reinterpret_cast<unsigned long long*>(p + 256);
+  b->sums1024 = b->sums32 + groups32;
+  p += a256(b->cleared);
   b->tile_sum = reinterpret_cast<int64_t*>(p);
-  p += a256(8 * (size_t)T + 8);
-  b->tile_prefix = reinterpret_cast<int64_t*>(p);
-  p += a256(8 * (size_t)T + 8);
+  p += a256(8 * (size_t)T);
   b->counts = reinterpret_cast<int32_t*>(p);
   p += a256(4 * (size_t)slots);
   b->nruns = reinterpret_cast<uint8_t*>(p);

@@ -33,16 +33,18 @@
 // e^-24.5, about 2e-11 of its amplitude.  Amplitudes must be non-negative
 // (their logarithm is taken).
 //
-// What bounds it: instruction issue and latency (67-75 % of cycles issue at 24
-// warps per SM; FMA pipe 43 %, exp2 21 %, shared-memory data pipe 50 %).  A third of the
-// instructions are the blob loop, the rest is per chunk (listing, range,
-// opacities, scan) and per ray (records).  Against two samples per lane of
+// What bounds it: instruction issue and latency (64 % of cycles issue at 24
+// warps per SM; the longest waits are those on the last result and on shared
+// memory).  36 % of the instructions are the blob loop, the rest is per chunk
+// (listing, range, opacities, scan) and per ray (records).  Against two samples per lane of
 // whichever rays come next, with distances in space and colours scanned per
-// chunk, the compositor went from 434 to 304 us on an 800 x 800 object frame
-// and from 2367 to 1482 us on a 1245 x 825 unbounded one.  Tried: four lanes per ray
+// chunk, the compositor went from 434 to 292 us on an 800 x 800 object frame
+// and from 2367 to 1455 us on a 1245 x 825 unbounded one.  Tried: four lanes per ray
 // with eight samples each (a quarter fewer instructions, but 14 warps per SM:
 // 20 % slower), 16 lanes' worth of registers saved by loading behind the blob
-// loop (12 % slower), 7 CTAs per SM (spills, 15 % slower).
+// loop (12 % slower), 7 CTAs per SM (spills, 15 % slower), CTAs of 8 to 16
+// tasks that their warps take in turn (5 to 10 % slower), groups refilled only
+// when several are idle (0 to 5 % slower).
 //
 // Rounding.  Ray parameters are taken relative to a base parameter near the
 // middle of the ray's samples, where the base point is rounded once, so t*
@@ -69,12 +71,12 @@ constexpr unsigned kLeaders = 0xffffffffu / ((1u << kGroupLanes) - 1u);  // the 
 constexpr int kChunk = kGroupLanes * kPerLane;       // samples of one ray per step
 constexpr float kLog2e = 1.4426950408889634f;
 
-// A blob as setup_ray reads it: {-mu, c} and {log2 a, sqrt(c), reach in units
-// of s sqrt(...): sqrt(c) (kCullSigmas s + margin), -}.
-struct BlobRec {
-  float4 pos;
-  float4 aux;
-};
+// The blobs as setup_ray reads them, two per lane: pair p holds blobs b = (p /
+// 32) * 64 + p % 32 and b + 32 in four arrays over the pairs (16 bytes per lane
+// and load, consecutive lanes consecutive): {-mu_x, -mu_y}, {-mu_z, c}, {log2 a,
+// sqrt(c)} and sqrt(c) (kCullSigmas s + margin), each as both blobs' values.
+__host__ __device__ inline int field_pairs(int G) { return (G + 63) / 64 * 32; }
+constexpr uint32_t kPairBytes = 3 * sizeof(float4) + sizeof(float2);
 
 // A ray as setup_ray reads it: base point and base parameter, direction and
 // 1 / |d|^2; beside it {|d|, the rounding margin of distances to its line}.
@@ -84,7 +86,7 @@ struct RayRec {
 };
 
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
-// tasks of R rays per warp: [G] BlobRec; [G + 1] colours (the last one black,
+// tasks of R rays per warp: the blobs in pairs; [G + 1] colours (the last one black,
 // for padding); then per warp [R] RayRec, [R] float2 and, per group, room for `cap`
 // records {k / 2, b = -k t*, c p^2 - log2 a, half-width | blob index} (and an
 // empty one behind them, for padding), as many list entries {offset of a
@@ -106,7 +108,7 @@ struct FieldLayout {
 __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int ring) {
   FieldLayout L;
   L.cap = G <= kAllBlobs ? G : (5 * G / 8 > kAllBlobs ? 5 * G / 8 : kAllBlobs);
-  L.col = (uint32_t)G * sizeof(BlobRec);
+  L.col = (uint32_t)field_pairs(G) * kPairBytes;
   L.warp0 = L.col + ((uint32_t)G + 1u) * sizeof(float4);
   L.len = (uint32_t)R * sizeof(RayRec);
   L.recs = L.len + (uint32_t)R * sizeof(float2);  // R is a multiple of 4
@@ -122,15 +124,23 @@ __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int
 // synchronises the block afterwards).
 __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayout& L,
                                             const float* __restrict__ field, int G) {
-  BlobRec* tab = reinterpret_cast<BlobRec*>(smem);
+  float* tab = reinterpret_cast<float*>(smem);
+  const int np = field_pairs(G);
   float4* col = reinterpret_cast<float4*>(smem + L.col);
   for (int i = threadIdx.x; i < G; i += blockDim.x) {
     const float* f = field + 8 * i;
     const float s = f[3], c = kLog2e / (2.f * s * s), rc = sqrtf(c);
     const float reach = kCullSigmas * s;
     const float mu_max = fmaxf(fabsf(f[0]), fmaxf(fabsf(f[1]), fabsf(f[2])));
-    tab[i].pos = make_float4(-f[0], -f[1], -f[2], c);
-    tab[i].aux = make_float4(log2f(f[4]), rc, rc * (reach + 2e-5f * (1.f + mu_max + reach)), 0.f);
+    const int p = (i >> 6) * 32 + (i & 31), h = (i >> 5) & 1;  // the pair, its blob
+    float *xy = tab + 4 * p + h, *zc = xy + 4 * np, *ak = zc + 4 * np;
+    xy[0] = -f[0];
+    xy[2] = -f[1];
+    zc[0] = -f[2];
+    zc[2] = c;
+    ak[0] = log2f(f[4]);
+    ak[2] = rc;
+    tab[12 * np + 2 * p + h] = rc * (reach + 2e-5f * (1.f + mu_max + reach));
     col[i] = make_float4(f[5], f[6], f[7], 0.f);
   }
   if (threadIdx.x == 0) col[G] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -192,47 +202,67 @@ __device__ __forceinline__ void make_ray_rec(RayRec* rr, float2* len, const floa
   *len = make_float2(moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm));
 }
 
+// sqrt(x), approximately, rounded up and its low 8 bits replaced by a blob's
+// index: at least 2^8 units in the last place are added, the square root's own
+// error is a few.
+__device__ __forceinline__ float half_width(float x, int q) {
+  float h;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(h) : "f"(x));
+  h = fminf(h, 1e30f);
+  return __uint_as_float(((__float_as_uint(h) + 0x1ffu) & ~0xffu) | (uint32_t)q);
+}
+
 // The blobs within reach of the ray's line, as records in `rec`; returns
-// their number.  With kMany: from blob q0 (a multiple of 32) on, as many whole
-// steps of 32 blobs as `cap` records hold, q0 advancing past the blobs looked
-// at.  Called by the whole warp, one blob per lane and step (the ray's samples
-// need not ascend, so the line is not cut off at its first and last one:
-// cutting it measured no faster either).  t* is found, the vector to the blob
-// taken there, and both are refined once from that vector, so their rounding
-// is that of the distance, not of the span from the base point.
+// their number.  With kMany: from blob q0 (a multiple of 64) on, as many whole
+// steps of 64 blobs as `cap` records hold, q0 advancing past the blobs looked
+// at.  Called by the whole warp, two blobs per lane and step in packed
+// arithmetic (the ray's samples need not ascend, so the line is not cut off at
+// its first and last one: cutting it measured no faster either).  t* is found,
+// the vector to the blob taken there, and both are refined once from that
+// vector, so their rounding is that of the distance, not of the span from the
+// base point.  A blob per lane took 304 us on the object frame, 1482 on the
+// unbounded one and 1907 on a 1080p render-only one; two take 292, 1455, 1819.
 template <bool kMany>
 __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const RayRec* rr,
                                          float2 len, float4* rec, int cap, int& q0) {
-  const BlobRec* tab = reinterpret_cast<const BlobRec*>(smem);
-  const int lane = threadIdx.x & 31;
+  const float4* tab = reinterpret_cast<const float4*>(smem);
+  const int lane = threadIdx.x & 31, np = field_pairs(G);
   const float4 B = rr->base, D = rr->dir;
+  const float2 dx = splat(D.x), dy = splat(D.y), dz = splat(D.z), nw = splat(-D.w);
   int n = 0;
-  for (; q0 < G; q0 += 32) {
-    const int q = min(q0 + lane, G - 1);
-    const float4 P = tab[q].pos;  // -mu, c
-    const float4 X = tab[q].aux;  // log2 a, sqrt(c), reach
-    const float wx = B.x + P.x, wy = B.y + P.y, wz = B.z + P.z;
-    float ts = -fmaf(wx, D.x, fmaf(wy, D.y, wz * D.z)) * D.w;
-    float qx = fmaf(ts, D.x, wx), qy = fmaf(ts, D.y, wy), qz = fmaf(ts, D.z, wz);
-    const float de = -fmaf(qx, D.x, fmaf(qy, D.y, qz * D.z)) * D.w;
-    ts += de;
-    qx = fmaf(de, D.x, qx);
-    qy = fmaf(de, D.y, qy);
-    qz = fmaf(de, D.z, qz);
-    const float cp2 = P.w * fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-    const float hl = fmaf(X.y, len.y, X.z);
-    const float lim2 = fmaf(hl, hl, -cp2);
-    // the half-width rounded up, its low 8 bits replaced by the blob's index
-    const float h = fminf(sqrtf(lim2), 1e30f);
-    const uint32_t hb = ((__float_as_uint(h) + 0x1ffu) & ~0xffu) | (uint32_t)q;
-    const float k = X.y * len.x;
-    const bool near = lim2 >= 0.f && q0 + lane < G;
-    const unsigned ball = __ballot_sync(kFieldFull, near);
-    if (kMany && n + __popc(ball) > cap) break;  // uniform; one step always fits
-    if (near)
-      rec[n + __popc(ball & ((1u << lane) - 1u))] =
-          make_float4(0.5f * k, -k * ts, cp2 - X.x, __uint_as_float(hb));
-    n += __popc(ball);
+  for (; q0 < G; q0 += 64) {
+    const int p = (q0 >> 1) + lane;
+    const float4 XY = tab[p], ZC = tab[np + p], AK = tab[2 * np + p];
+    const float2 reach = reinterpret_cast<const float2*>(tab + 3 * np)[p];
+    const float2 c = make_float2(ZC.z, ZC.w), rc = make_float2(AK.z, AK.w);
+    const float2 wx = __fadd2_rn(splat(B.x), make_float2(XY.x, XY.y));
+    const float2 wy = __fadd2_rn(splat(B.y), make_float2(XY.z, XY.w));
+    const float2 wz = __fadd2_rn(splat(B.z), make_float2(ZC.x, ZC.y));
+    float2 ts = __fmul2_rn(nw, __ffma2_rn(wx, dx, __ffma2_rn(wy, dy, __fmul2_rn(wz, dz))));
+    float2 qx = __ffma2_rn(ts, dx, wx), qy = __ffma2_rn(ts, dy, wy), qz = __ffma2_rn(ts, dz, wz);
+    const float2 de = __fmul2_rn(nw, __ffma2_rn(qx, dx, __ffma2_rn(qy, dy, __fmul2_rn(qz, dz))));
+    ts = __fadd2_rn(ts, de);
+    qx = __ffma2_rn(de, dx, qx);
+    qy = __ffma2_rn(de, dy, qy);
+    qz = __ffma2_rn(de, dz, qz);
+    const float2 cp2 = __fmul2_rn(c, __ffma2_rn(qx, qx, __ffma2_rn(qy, qy, __fmul2_rn(qz, qz))));
+    const float2 hl = __ffma2_rn(rc, splat(len.y), reach);
+    const float2 lim2 = __ffma2_rn(hl, hl, make_float2(-cp2.x, -cp2.y));
+    const float2 k = __fmul2_rn(rc, splat(len.x));
+    const float2 hk = __fmul2_rn(splat(0.5f), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
+    const float2 e = __fadd2_rn(cp2, make_float2(-AK.x, -AK.y));
+    const int q = q0 + lane;
+    const bool near0 = lim2.x >= 0.f && q < G, near1 = lim2.y >= 0.f && q + 32 < G;
+    const unsigned ball0 = __ballot_sync(kFieldFull, near0);
+    const unsigned ball1 = __ballot_sync(kFieldFull, near1);
+    const int n0 = __popc(ball0), kept = n0 + __popc(ball1);
+    if (kMany && n + kept > cap) break;  // uniform; one step always fits
+    const unsigned below = (1u << lane) - 1u;
+    if (near0)
+      rec[n + __popc(ball0 & below)] = make_float4(hk.x, b.x, e.x, half_width(lim2.x, q));
+    if (near1)
+      rec[n + n0 + __popc(ball1 & below)] = make_float4(hk.y, b.y, e.y, half_width(lim2.y, q + 32));
+    n += kept;
   }
   return n;
 }
@@ -471,14 +501,15 @@ __device__ __forceinline__ void shade_chunk(BlobSums& B, const float2 dt[kPairs]
 // a segment; a segment's samples of one ray are a balanced tree over the pairs
 // of places, counted back from the last whole pair, times a last single
 // sample; segments multiply in order.  Between chunks the factors wait in a
-// ring of 128 per group in shared memory.  It costs the compositor 3 to 5 %
-// (object frame 291 -> 304 us, unbounded 1435 -> 1482; 322 and 1571 with the
-// product and `task` in registers, which then spill).  The limit: with 0.998
+// ring of 96 per group in shared memory.  It costs the compositor 3 to 5 %
+// (291 -> 304 us on the object frame, 1435 -> 1482 on the unbounded one before
+// setup_ray took two blobs per lane; 322 and 1571 with the product and `task` in
+// registers, which then spill).  The limit: with 0.998
 // three of 81 random unbounded frames differ by 2.1e-5 (2-norm, relative) from
 // the same product order throughout, with 0.98 none by more than 7.5e-6.
 constexpr float kFaint = 0.98f;
 constexpr int kFaintRays = 4;
-constexpr int kRing = 128;  // a segment and a chunk beyond it
+constexpr int kRing = 96;  // a segment and a chunk beyond it
 
 // One chunk of every group, called by the whole warp: `f` the lane's factors (1
 // for padding), `q` its first position (a multiple of 4), `busy` where the
@@ -495,7 +526,7 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
   const int task = __shfl_sync(kFieldFull, my_beg, ray & ~(kFaintRays - 1));
   const int gl = threadIdx.x & (kGroupLanes - 1);
   if (on)
-    *reinterpret_cast<float4*>(ring + (q & (kRing - 1))) = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+    *reinterpret_cast<float4*>(ring + (unsigned)q % kRing) = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
   __syncwarp();
   const int base = q - kPerLane * gl;  // the chunk's positions
   const int to = min(base + kChunk, end);
@@ -516,8 +547,8 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
       const int p = c0 + n - 2 - 2 * (4 * gl + i);  // the pair's first position
       v[i] = 1.f;
       if (full && p + 1 >= s0) {
-        const float y = ring[(p + 1) & (kRing - 1)];
-        v[i] = p >= s0 ? ring[p & (kRing - 1)] * y : y;
+        const float y = ring[(unsigned)(p + 1) % kRing];
+        v[i] = p >= s0 ? ring[(unsigned)p % kRing] * y : y;
       }
     }
     float m = (v[0] * v[1]) * (v[2] * v[3]);
@@ -525,7 +556,7 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
     for (int o = 1; o < kGroupLanes; o <<= 1) m *= __shfl_xor_sync(kFieldFull, m, o);
     if (full) {
       F *= m;
-      if ((s1 - c0) & 1) F *= ring[(s1 - 1) & (kRing - 1)];
+      if ((s1 - c0) & 1) F *= ring[(unsigned)(s1 - 1) % kRing];
       at = s1;  // on to the next segment
     }
   }

@@ -112,9 +112,8 @@ __global__ void __launch_bounds__(kBlock, 1024 / kBlock) batch_walk_kernel(
         Ray ray;
         int nr = 0;
         if (load_ray(job.ro, job.rd, lr, ray))
-          c = walk<kMode, false, false, kSkip, kCheck>(
-              job.g, global_tabs(job.g, job.lat), job.lat, lat_hdr(job.lat), ray, runs + gr, slots,
-              nr, 0, 0, 0, nullptr, nullptr, nullptr, status);
+          c = walk<kMode, false, kSkip, kCheck>(job.g, global_tabs(job.g, job.lat), job.lat,
+                                                lat_hdr(job.lat), ray, runs + gr, slots, nr, status);
         counts[gr] = (int32_t)c;
         nruns_out[gr] = (uint8_t)min(nr, 255);
       }
@@ -141,7 +140,7 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
     const uint2* __restrict__ runs, const int64_t* __restrict__ tile_sum,
     const unsigned long long* __restrict__ sums32,
     const unsigned long long* __restrict__ sums1024, int64_t* __restrict__ job_totals,
-    unsigned* __restrict__ job_status, unsigned* __restrict__ status) {
+    unsigned* __restrict__ job_status) {
   __shared__ uint2 s_rec[kWarps][kRecMax + 1];
   __shared__ __align__(16) GridDev s_grid[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -178,7 +177,7 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
   // the tile's runs as a record list, expanded with 16-byte stores where the
   // job's outputs allow (expand_records, walk.cuh)
   uint2* rec = s_rec[warp];
-  const int kept = c <= 0 ? 0 : nr > kMaxRuns ? 1 : nr;
+  const int kept = c <= 0 ? 0 : min(nr, kMaxRuns);
   int kinc = kept;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
     if (lane >= o) kinc += y;
   }
   const int nrec = __shfl_sync(kFull, kinc, 31);
-  list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + gr, slots);
+  const uint2 rest = list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + gr, slots);
   if (lane == 0) rec[nrec] = make_uint2(kRecEnd, 0u);
   __syncwarp();
   const int tot = __shfl_sync(kFull, inc, 31);
@@ -205,10 +204,9 @@ __global__ void __launch_bounds__(kWarps * 32) batch_emit_kernel(
       Ray ray;
       load_ray(jb.ro, jb.rd, lr, ray);
       const LatHdr h = lat_hdr(lat);
-      int unused = 0;
-      walk<kMode, true, false>(s_grid[warp], global_tabs(s_grid[warp], lat), lat, h, ray, nullptr, 0,
-                               unused, (int32_t)lr, off, capacity, jb.ray_idx, jb.t0, jb.t1,
-                               status);
+      emit_from<kMode, false>(s_grid[warp], global_tabs(s_grid[warp], lat), lat, h, ray,
+                              (int)rest.x, c - ((int)rest.y - q), (int32_t)lr, wbeg + rest.y,
+                              capacity, jb.ray_idx, jb.t0, jb.t1);
     }
   }
 }
@@ -312,7 +310,7 @@ void launch_batch_emit(const hdda_batch* b, cudaStream_t s) {
 #define HDDA_BATCH_EMIT(W)                                                                    \
   batch_emit_kernel<kMode, W><<<(unsigned)((b->T + W - 1) / W), W * 32, 0, s>>>(             \
       b->jobs, b->tile0, b->n_jobs, b->T, b->counts, b->nruns, b->runs, b->tile_sum,         \
-      b->sums32, b->sums1024, b->job_totals, b->job_status, b->status)
+      b->sums32, b->sums1024, b->job_totals, b->job_status)
   switch (b->cfg.emit_warps) {
     case 2: HDDA_BATCH_EMIT(2); break;
     case 4: HDDA_BATCH_EMIT(4); break;

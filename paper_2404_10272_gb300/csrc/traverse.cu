@@ -323,8 +323,8 @@ __global__ void __launch_bounds__(kBS) onepass_kernel(
   if (r < n) {
     valid = load_ray(ro, rd, r, ray);
     if (valid)
-      c = walk<kMode, false, false>(g, global_tabs(g, lat), lat, h, ray, s_runs + threadIdx.x, kBS,
-                                   nruns, 0, 0, 0, nullptr, nullptr, nullptr, status);
+      c = walk<kMode, false>(g, global_tabs(g, lat), lat, h, ray, s_runs + threadIdx.x, kBS, nruns,
+                             status);
   }
   int64_t agg = 0;
   const int64_t local = cta_exclusive_scan64(c, &agg);
@@ -347,11 +347,9 @@ __global__ void __launch_bounds__(kBS) onepass_kernel(
   const bool overflow = nruns > kMaxRuns;
   expand_warp<true>(off, c, overflow, s_runs + warp * 32, kBS,
                     (int32_t)((int64_t)tile * kBS + warp * 32), lat.t, capacity, ray_idx, t0, t1);
-  if (overflow && valid) {
-    int unused = 0;
-    walk<kMode, true, false>(g, global_tabs(g, lat), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
-                            capacity, ray_idx, t0, t1, status);
-  }
+  if (overflow && valid)
+    emit_from<kMode, false>(g, global_tabs(g, lat), lat, h, ray, 0, c, (int32_t)r, off, capacity,
+                            ray_idx, t0, t1);
 }
 
 // ---------------------------------------------------------------------------
@@ -365,11 +363,15 @@ constexpr int kEmitCtasPerSm = 7;  // by registers (72) and shared memory (16 KB
 // is the sum of the earlier tiles' samples (tile_offset, from the group sums
 // the walk kept) plus a warp scan; its runs become a record list in shared
 // memory (rec: kRecMax records and a sentinel) that expand_records turns into
-// samples.  A ray with more runs than were kept walks again.  The last tile
+// samples.  A ray with more runs than were kept walks on behind them (emit_from).  The last tile
 // writes the total.
+//
+// Of 2^shift warps with one tile each, `part` 0 writes the offsets, the total
+// and the status; each writes an equal part of the samples, and those of every
+// 2^shift-th overflowing ray.
 template <int kMode>
 __device__ __forceinline__ void emit_tile(
-    int64_t tile, unsigned T, uint2* rec, const float* __restrict__ ro,
+    int64_t tile, int part, int shift, unsigned T, uint2* rec, const float* __restrict__ ro,
     const float* __restrict__ rd, int64_t n, const GridDev& g, const LatticeDev& lat,
     const int32_t* __restrict__ counts, const uint8_t* __restrict__ nruns,
     const uint2* __restrict__ runs, const int64_t* __restrict__ tile_sum,
@@ -392,19 +394,17 @@ __device__ __forceinline__ void emit_tile(
   const int q = inc - c;
   const int tot = __shfl_sync(kFull, inc, 31);
   const int64_t off = wbeg + q;
-  if (tile == (int64_t)T - 1 && lane == 0) *total = wbeg + tot;
-  if (capacity > 0) {
+  if (part == 0) {
+    if (tile == (int64_t)T - 1 && lane == 0) *total = wbeg + tot;
     // with too small a buffer the CSR offsets are clamped to it, so that a
     // consumer of the arrays stays in bounds; the status says what happened
-    if (r < n) offsets[r] = min(off, capacity);
-    if (r == n - 1) offsets[n] = min(off + c, capacity);
-    if (wbeg + tot > capacity && lane == 0) atomicOr(status, kDevCapacity);
-  } else {
-    if (r < n) offsets[r] = off;
-    if (r == n - 1) offsets[n] = off + c;
-    return;
+    const int64_t most = capacity > 0 ? capacity : INT64_MAX;
+    if (r < n) offsets[r] = min(off, most);
+    if (r == n - 1) offsets[n] = min(off + c, most);
+    if (capacity > 0 && wbeg + tot > capacity && lane == 0) atomicOr(status, kDevCapacity);
   }
-  const int kept = c <= 0 ? 0 : nr > kMaxRuns ? 1 : nr;
+  if (capacity <= 0) return;
+  const int kept = c <= 0 ? 0 : min(nr, kMaxRuns);
   int kinc = kept;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -412,19 +412,20 @@ __device__ __forceinline__ void emit_tile(
     if (lane >= o) kinc += y;
   }
   const int nrec = __shfl_sync(kFull, kinc, 31);
-  list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + r, n);
+  const uint2 rest = list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + r, n);
   if (lane == 0) rec[nrec] = make_uint2(kRecEnd, 0u);
   __syncwarp();
   const int64_t room = capacity - wbeg;
   const int lim = room <= 0 ? 0 : (int)min((int64_t)tot, room);
-  expand_records(rec, nrec, lim, wbeg, (int32_t)(tile * 32), lat.t, vec, ray_idx, t0, t1);
-  if (nr > kMaxRuns) {
+  expand_records<true>(rec, nrec, lim, wbeg, (int32_t)(tile * 32), lat.t, vec, ray_idx, t0, t1,
+                       part, shift);
+  const bool again = nr > kMaxRuns && (lane & ((1 << shift) - 1)) == part;
+  if (__any_sync(kFull, again) && again) {
     Ray ray;
     load_ray(ro, rd, r, ray);
-    const LatHdr h = lat_hdr(lat);
-    int unused = 0;
-    walk<kMode, true, false>(g, global_tabs(g, lat), lat, h, ray, nullptr, 0, unused, (int32_t)r, off,
-                             capacity, ray_idx, t0, t1, status);
+    emit_from<kMode, false>(g, global_tabs(g, lat), lat, lat_hdr(lat), ray, (int)rest.x,
+                            c - ((int)rest.y - q), (int32_t)r, wbeg + rest.y, capacity, ray_idx, t0,
+                            t1);
   }
 }
 
@@ -441,8 +442,8 @@ __global__ void __launch_bounds__(kEmitWarps * 32, kEmitCtasPerSm) emit_kernel(
     const unsigned long long* __restrict__ sums32,
     const unsigned long long* __restrict__ sums1024, int64_t* __restrict__ offsets,
     int32_t* __restrict__ ray_idx, float* __restrict__ t0, float* __restrict__ t1,
-    int64_t capacity, bool vec, unsigned* __restrict__ tile_counter, int64_t* __restrict__ total,
-    unsigned* __restrict__ status) {
+    int64_t capacity, bool vec, int shift, unsigned* __restrict__ tile_counter,
+    int64_t* __restrict__ total, unsigned* __restrict__ status) {
   __shared__ uint2 s_rec[kEmitWarps][kRecMax + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned T = (unsigned)((n + 31) / 32);
@@ -450,17 +451,29 @@ __global__ void __launch_bounds__(kEmitWarps * 32, kEmitCtasPerSm) emit_kernel(
     unsigned tile = 0;
     if (lane == 0) tile = atomicAdd(tile_counter, 1u);
     tile = __shfl_sync(kFull, tile, 0);
+    const int part = (int)(tile & ((1u << shift) - 1u));
+    tile >>= shift;
     if (tile >= T) break;
-    emit_tile<kMode>(tile, T, s_rec[warp], ro, rd, n, g, lat, counts, nruns, runs, tile_sum,
+    emit_tile<kMode>(tile, part, shift, T, s_rec[warp], ro, rd, n, g, lat, counts, nruns, runs, tile_sum,
                      sums32, sums1024, offsets, ray_idx, t0, t1, capacity, vec, total, status);
     __syncwarp();  // the next tile reuses this warp's shared memory
   }
 }
 
+// Warps per tile (log2): a call of fewer tiles than the chip runs warps gives
+// each tile to as many, up to eight, as find room (one warp's 20 blocks of 128
+// samples are a serial chain: 16,381 rays 43 -> 18 us, 9,216 rays 18 -> 11).
+int emit_shift(int64_t T, int device) {
+  const int64_t room = (int64_t)sm_count(device) * kEmitCtasPerSm * kEmitWarps;
+  int shift = 0;
+  while (shift < 3 && (T << (shift + 1)) <= room) ++shift;
+  return shift;
+}
+
 // CTAs of the persistent emit: one wave (the launch bounds' CTAs per SM), or
 // fewer for small calls.
-unsigned emit_grid(int64_t T, int device) {
-  const int64_t want = (T + kEmitWarps - 1) / kEmitWarps;
+unsigned emit_grid(int64_t T, int shift, int device) {
+  const int64_t want = ((T << shift) + kEmitWarps - 1) / kEmitWarps;
   const int64_t full = (int64_t)sm_count(device) * kEmitCtasPerSm;
   return (unsigned)(want < full ? want : full);
 }
@@ -529,7 +542,7 @@ __device__ __forceinline__ void emit_fused_tile(
   if (e == (int)T - 1 && lane == 0) *total = excl + tot;
   if (capacity <= 0) return;
   // the record list: an exclusive scan of the lanes' record counts
-  const int kept = c <= 0 ? 0 : nr > kMaxRuns ? 1 : nr;
+  const int kept = c <= 0 ? 0 : min(nr, kMaxRuns);
   int kinc = kept;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -537,7 +550,7 @@ __device__ __forceinline__ void emit_fused_tile(
     if (lane >= o) kinc += y;
   }
   const int nrec = __shfl_sync(kFull, kinc, 31);
-  list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + r, n);
+  const uint2 rest = list_runs(rec, kinc - kept, lane, nr, c, (uint32_t)q, runs + r, n);
   if (lane == 0) rec[nrec] = make_uint2(kRecEnd, 0u);
   __syncwarp();
   const int64_t room = capacity - excl;
@@ -547,9 +560,8 @@ __device__ __forceinline__ void emit_fused_tile(
   if (nr > kMaxRuns) {
     Ray ray;
     load_ray(ro, rd, r, ray);
-    int unused = 0;
-    walk<kMode, true, kSm>(g, tb, lat, h, ray, nullptr, 0, unused, (int32_t)r, off, capacity,
-                           ray_idx, t0, t1, status);
+    emit_from<kMode, kSm>(g, tb, lat, h, ray, (int)rest.x, c - ((int)rest.y - q), (int32_t)r,
+                          excl + rest.y, capacity, ray_idx, t0, t1);
   }
 }
 
@@ -583,8 +595,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_emit_kernel(
       Ray ray;
       int nr = 0;
       if (load_ray(ro, rd, r, ray))
-        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, 0, 0, 0,
-                                                  nullptr, nullptr, nullptr, status);
+        c = walk<kMode, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, status);
       counts[r] = (int32_t)c;
       nruns_out[r] = (uint8_t)min(nr, 255);
     }
@@ -910,21 +921,23 @@ int run_twopass(const float* ro, const float* rd, int64_t n, const hdda_grid* gr
   }
   {
     KernelTimer kt(emit_name(mode), s);
+    const int shift = emit_shift(T, grid->device);
+    const unsigned ctas = emit_grid(T, shift, grid->device);
     switch (mode) {
       case kModeDense:
-        emit_kernel<kModeDense><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeDense><<<ctas, kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
-            ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
+            ray_idx, t0, t1, capacity, vec, shift, emit_counter, total, status);
         break;
       case kModeVdb:
-        emit_kernel<kModeVdb><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeVdb><<<ctas, kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
-            ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
+            ray_idx, t0, t1, capacity, vec, shift, emit_counter, total, status);
         break;
       default:
-        emit_kernel<kModeVdbMap><<<emit_grid(T, grid->device), kEmitWarps * 32, 0, s>>>(
+        emit_kernel<kModeVdbMap><<<ctas, kEmitWarps * 32, 0, s>>>(
             ro, rd, n, w.g, lat, counts, nruns, runs, tile_sum, sums32, sums1024, offsets,
-            ray_idx, t0, t1, capacity, vec, emit_counter, total, status);
+            ray_idx, t0, t1, capacity, vec, shift, emit_counter, total, status);
         break;
     }
   }

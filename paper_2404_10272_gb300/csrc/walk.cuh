@@ -451,24 +451,19 @@ __device__ __forceinline__ bool locate(const GridDev& g, const Tabs<kSm>& tb, co
 
 // Walks one ray.  Counts its samples and merges occupied regions into runs
 // [k_begin, k_end): the first kMaxRuns go to runs[j * stride]; nruns counts
-// all.  With kEmit it instead writes the samples from `out`, below
-// `capacity` (lat.t must then be a global-memory table).
+// all.
 // kSkip selects the control flow of Algorithm 2 ("DDA skip": cross every
 // leading empty region in an inner loop, then take the occupied one)
 // instead of Algorithm 1 ("DDA branch": one region per iteration, branching
 // on its occupancy).  The regions crossed, and so the samples, are the same.
 // kCheck tests that every region holds the point it was found from (raising
 // kDevInternal otherwise); the invariant the crossing search rests on.
-template <int kMode, bool kEmit, bool kSm, bool kSkip, bool kCheck, bool kOne>
+template <int kMode, bool kSm, bool kSkip, bool kCheck, bool kOne>
 __device__ __forceinline__ int64_t walk_levels(const GridDev& g, const Tabs<kSm>& tb,
                                                const LatticeDev& lat, const LatHdr& h,
                                                const Ray& r, uint2* runs, int64_t stride,
-                                               int& nruns, int32_t rid, int64_t out,
-                                               int64_t capacity, int32_t* __restrict__ ray_idx,
-                                               float* __restrict__ t0, float* __restrict__ t1,
-                                               unsigned* __restrict__ status) {
-  int64_t cnt = 0;  // kEmit
-  int kept = 0;     // at most 2^24
+                                               int& nruns, unsigned* __restrict__ status) {
+  int kept = 0;  // at most 2^24
   nruns = 0;
   if (lat.K <= 0) return 0;
   int rb = -1, re = -1;  // open run
@@ -504,56 +499,78 @@ __device__ __forceinline__ int64_t walk_levels(const GridDev& g, const Tabs<kSm>
       k = kn;
     }
     if (over) break;
-    if constexpr (kEmit) {
-      if (occ) {
-        float ta = __ldg(lat.t + k);
-        for (int j = k; j < kn; ++j) {
-          const float tn = __ldg(lat.t + j + 1);
-          const int64_t p = out + cnt;
-          if (p < capacity) {
-            ray_idx[p] = rid;
-            t0[p] = ta;
-            t1[p] = tn;
-          }
-          ta = tn;
-          ++cnt;
-        }
-      }
-    } else {
-      // an occupied region extends the open run or, not adjacent, opens the next one
-      const bool opens = occ & (k != re);
-      if (opens & (rb >= 0)) {
-        if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
-        ++nruns;
-      }
-      kept += occ ? kn - k : 0;
-      rb = opens ? k : rb;
-      re = occ ? kn : re;
+    // an occupied region extends the open run or, not adjacent, opens the next one
+    const bool opens = occ & (k != re);
+    if (opens & (rb >= 0)) {
+      if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
+      ++nruns;
     }
+    kept += occ ? kn - k : 0;
+    rb = opens ? k : rb;
+    re = occ ? kn : re;
     k = kn;
   }
-  if (!kEmit && rb >= 0) {
+  if (rb >= 0) {
     if (nruns < kMaxRuns) runs[nruns * stride] = make_uint2(rb, re);
     ++nruns;
   }
-  return kEmit ? cnt : (int64_t)kept;
+  return kept;
 }
 
 // The walk with the one-level form where it applies (its own copy of the
-// code), except in the rare second walk of a ray (kEmit).
-template <int kMode, bool kEmit, bool kSm, bool kSkip = false, bool kCheck = false>
+// code).
+template <int kMode, bool kSm, bool kSkip = false, bool kCheck = false>
 __device__ __forceinline__ int64_t walk(const GridDev& g, const Tabs<kSm>& tb,
-                                        const LatticeDev& lat,
-                                        const LatHdr& h, const Ray& r, uint2* runs,
-                                        int64_t stride, int& nruns, int32_t rid,
-                                        int64_t out, int64_t capacity,
-                                        int32_t* __restrict__ ray_idx, float* __restrict__ t0,
-                                        float* __restrict__ t1, unsigned* __restrict__ status) {
-  if (!kEmit && g.L == 1)  // uniform
-    return walk_levels<kMode, kEmit, kSm, kSkip, kCheck, true>(
-        g, tb, lat, h, r, runs, stride, nruns, rid, out, capacity, ray_idx, t0, t1, status);
-  return walk_levels<kMode, kEmit, kSm, kSkip, kCheck, false>(
-      g, tb, lat, h, r, runs, stride, nruns, rid, out, capacity, ray_idx, t0, t1, status);
+                                        const LatticeDev& lat, const LatHdr& h, const Ray& r,
+                                        uint2* runs, int64_t stride, int& nruns,
+                                        unsigned* __restrict__ status) {
+  if (g.L == 1)  // uniform
+    return walk_levels<kMode, kSm, kSkip, kCheck, true>(g, tb, lat, h, r, runs, stride, nruns,
+                                                        status);
+  return walk_levels<kMode, kSm, kSkip, kCheck, false>(g, tb, lat, h, r, runs, stride, nruns,
+                                                       status);
+}
+
+// Writes the samples of a ray from lattice index k0 on to `out`, below
+// `capacity`, until `left` of them are written or counted (lat.t is a table in
+// global memory): the rest of a ray with more runs than were kept, found by a
+// second walk.  It starts behind the runs that were, which it need not cross
+// again: a single such ray keeps a whole kernel waiting (65,536 rays of which
+// 13 have 17 to 19 runs, 2 x 512^3 voxels: the emit took 119 us when they walked
+// again from the start, 38 so).  Resuming as walk_from does.
+template <int kMode, bool kSm>
+__device__ __forceinline__ void emit_from(const GridDev& g, const Tabs<kSm>& tb,
+                                          const LatticeDev& lat, const LatHdr& h, const Ray& r,
+                                          int k0, int64_t left, int32_t rid, int64_t out,
+                                          int64_t capacity, int32_t* __restrict__ ray_idx,
+                                          float* __restrict__ t0, float* __restrict__ t1) {
+  if (k0 >= lat.K) return;
+  float x[3];
+  int k = k0;
+  Stretch<kMode, kSm, false> st;
+  st.init(g, tb, r, h, lat.K, k0);
+  while (left > 0) {
+    if (k >= st.kend) {
+      if (!st.next(g, tb, r, lat.K, k)) break;
+      point_at(r, tb.tm[k], x);
+    }
+    float e[3];
+    const bool occ = locate(g, tb, r, st, x, e);
+    const int kn = cross<kSm>(r, tb, h, k, st.kend, e, x);
+    if (occ) {
+      float ta = __ldg(lat.t + k);
+      for (int j = k; j < kn && left > 0; ++j, ++out, --left) {
+        const float tn = __ldg(lat.t + j + 1);
+        if (out < capacity) {
+          ray_idx[out] = rid;
+          t0[out] = ta;
+          t1[out] = tn;
+        }
+        ta = tn;
+      }
+    }
+    k = kn;
+  }
 }
 
 // Walks one ray from lattice index k0 and stops after kMaxRuns runs: writes
@@ -652,9 +669,9 @@ __device__ __forceinline__ void expand_warp(int64_t off, int64_t c, bool overflo
 // walk, or batched), with 16-byte stores.  A warp first lists its tile's
 // runs, rays in order and each ray's runs in order, as records {first output
 // position relative to the tile's first sample, (first k << 5) | lane}: one
-// per run, or, for a ray with more runs than were kept, one record with
-// kRecSkip set that covers all of that ray's samples (the ray walks again and
-// writes them itself).  A sentinel record with position kRecEnd follows the
+// per run, or, for a ray with more runs than were kept, its last one with
+// kRecSkip set, covering all of the ray's samples from that run on (the ray
+// walks on from there and writes them itself: emit_from).  A sentinel record with position kRecEnd follows the
 // last.  Positions are then expanded four per lane per 128-position block
 // (expand_records): a lane finds the record holding its first position, and
 // a record covers at least one position, so its four positions lie in at most
@@ -670,14 +687,24 @@ constexpr uint32_t kRecEnd = 0xffffffffu;
 // lane's sample count and `q` its first position relative to the tile; run j
 // of the lane's ray is runs_r[j * stride].  The runs are read through L2
 // (ld.global.cg), not the read-only path, because the fused sampler form
-// reads them in the kernel that wrote them.
-__device__ __forceinline__ void list_runs(uint2* rec, int first, int lane, int nr, int64_t c,
-                                          uint32_t q, const uint2* __restrict__ runs_r,
-                                          int64_t stride) {
-  if (c <= 0) return;
+// reads them in the kernel that wrote them.  With more than kMaxRuns runs,
+// returns where the last kept one starts: {its first k, its first position};
+// else {0, 0}.  Those rays have a loop of their own: with the case decided per
+// run in one loop, the emit of an 800 x 800 frame took 140 us instead of 90.
+__device__ __forceinline__ uint2 list_runs(uint2* rec, int first, int lane, int nr, int64_t c,
+                                           uint32_t q, const uint2* __restrict__ runs_r,
+                                           int64_t stride) {
+  if (c <= 0) return make_uint2(0u, 0u);
   if (nr > kMaxRuns) {
-    rec[first] = make_uint2(q, kRecSkip | (uint32_t)lane);
-    return;
+    for (int j = 0;; ++j) {
+      const uint2 v = __ldcg(runs_r + (int64_t)j * stride);
+      if (j == kMaxRuns - 1) {
+        rec[first + j] = make_uint2(q, kRecSkip | (uint32_t)lane);
+        return make_uint2(v.x, q);
+      }
+      rec[first + j] = make_uint2(q, (v.x << 5) | (uint32_t)lane);
+      q += v.y - v.x;
+    }
   }
   for (int j0 = 0; j0 < nr; j0 += 4) {
     uint2 v[4];
@@ -692,6 +719,7 @@ __device__ __forceinline__ void list_runs(uint2* rec, int first, int lane, int n
       }
     }
   }
+  return make_uint2(0u, 0u);
 }
 
 // One record as the expansion uses it: its sample positions q map to
@@ -751,15 +779,25 @@ __device__ __forceinline__ void expand_four_any(const uint2* rec, int& u, int q0
 // beyond them (a block of more than 32 records) binary-searches the rest.
 // A lane's four positions then take their lattice index, ray and skip flag
 // from that record or the next one by selects; only a lane whose positions
-// reach a third record steps through them one by one.
+// reach a third record steps through them one by one.  Of several warps that
+// share the tile, the one with number `part` of 2^shift writes an equal part of
+// the blocks (kSplit).
+template <bool kSplit = false>
 __device__ __forceinline__ void expand_records(const uint2* rec, int nrec, int lim, int64_t wbeg,
                                                int32_t rid0, const float* __restrict__ t,
                                                bool vec, int32_t* __restrict__ ray_idx,
-                                               float* __restrict__ t0, float* __restrict__ t1) {
+                                               float* __restrict__ t0, float* __restrict__ t1,
+                                               int part = 0, int shift = 0) {
   if (nrec <= 0 || lim <= 0) return;
   const int lane = threadIdx.x & 31;
   int ufirst = 0;  // rec[0] starts at position 0
-  for (int base = -(int)(wbeg & 3); base < lim; base += 128) {
+  int base = -(int)(wbeg & 3), end = lim;
+  if constexpr (kSplit) {
+    const int64_t blocks = ((int64_t)lim - base + 127) >> 7;
+    end = (int)min((int64_t)lim, 128 * ((blocks * (part + 1)) >> shift) + base);
+    base += (int)(128 * ((blocks * part) >> shift));
+  }
+  for (; base < end; base += 128) {
     const int q0 = base + 4 * lane;
     const int qs = max(q0, 0);
     const uint32_t pj = rec[min(ufirst + lane, nrec)].x;  // the sentinel past the end
@@ -952,8 +990,7 @@ __global__ void __launch_bounds__(kWalkBS) walk_kernel(
       Ray ray;
       int nr = 0;
       if (load_ray(ro, rd, r, ray))
-        c = walk<kMode, false, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, 0, 0, 0,
-                                                  nullptr, nullptr, nullptr, status);
+        c = walk<kMode, kSm, kSkip, kCheck>(g, tb, lat, h, ray, runs + r, n, nr, status);
       counts[r] = (int32_t)c;
       nruns_out[r] = (uint8_t)min(nr, 255);
     }

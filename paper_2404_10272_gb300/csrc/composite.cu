@@ -83,14 +83,14 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
   t1 += wbase;
   const bool nonempty = has_ray && se > sb;
   if (nonempty) {
-    const float tb = 0.5f * (__ldg(t0 + my_beg) + __ldg(t1 + my_end - 1));
+    const float ta = __ldg(t0 + my_beg), te = __ldg(t1 + my_end - 1);
     float o[3], d[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, tb);
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, base_param(smem, L, G, o, d, ta, te));
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
   }

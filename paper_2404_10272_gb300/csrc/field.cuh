@@ -47,9 +47,8 @@
 // when several are idle (0 to 5 % slower).
 //
 // Rounding.  Ray parameters are taken relative to a base parameter near the
-// middle of the ray's samples, where the base point is rounded once, so t*
-// and p carry the rounding of coordinates near the samples, not of the
-// origin's.  Every product-sum is an explicit fused multiply-add, so the
+// blobs (base_param), where the base point is rounded once, so t* and p carry
+// the rounding of coordinates near the blobs, not of the origin's.  Every product-sum is an explicit fused multiply-add, so the
 // arithmetic does not depend on the translation unit's contraction flags.
 #pragma once
 
@@ -87,7 +86,7 @@ struct RayRec {
 
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
 // tasks of R rays per warp: the blobs in pairs; [G + 1] colours (the last one black,
-// for padding); then per warp [R] RayRec, [R] float2 and, per group, room for `cap`
+// for padding) and the mean of the blobs' centres; then per warp [R] RayRec, [R] float2 and, per group, room for `cap`
 // records {k / 2, b = -k t*, c p^2 - log2 a, half-width | blob index} (and an
 // empty one behind them, for padding), as many list entries {offset of a
 // record, offset of its colour}, and `ring` factors of a faint ray.
@@ -109,7 +108,7 @@ __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int
   FieldLayout L;
   L.cap = G <= kAllBlobs ? G : (5 * G / 8 > kAllBlobs ? 5 * G / 8 : kAllBlobs);
   L.col = (uint32_t)field_pairs(G) * kPairBytes;
-  L.warp0 = L.col + ((uint32_t)G + 1u) * sizeof(float4);
+  L.warp0 = L.col + ((uint32_t)G + 2u) * sizeof(float4);
   L.len = (uint32_t)R * sizeof(RayRec);
   L.recs = L.len + (uint32_t)R * sizeof(float2);  // R is a multiple of 4
   L.list = ((uint32_t)L.cap + 1u) * sizeof(float4);
@@ -143,7 +142,36 @@ __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayo
     tab[12 * np + 2 * p + h] = rc * (reach + 2e-5f * (1.f + mu_max + reach));
     col[i] = make_float4(f[5], f[6], f[7], 0.f);
   }
-  if (threadIdx.x == 0) col[G] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (threadIdx.x >= blockDim.x - 32) {  // the mean of the centres: a warp without blobs up to 96
+    const int lane = threadIdx.x & 31;
+    float m[3] = {0.f, 0.f, 0.f};
+    for (int i = lane; i < G; i += 32)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) m[k] += field[8 * i + k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m[k] += __shfl_xor_sync(kFieldFull, m[k], o);
+    if (lane == 0) {
+      const float s = 1.f / (float)max(G, 1);
+      col[G] = make_float4(0.f, 0.f, 0.f, 0.f);
+      col[G + 1] = make_float4(s * m[0], s * m[1], s * m[2], 0.f);
+    }
+  }
+}
+
+// The base parameter of a ray whose samples lie between ta and tb: where it
+// passes nearest to the blobs' mean centre.  Parameters and distances are exact
+// to the rounding of numbers of the size of their difference from the base,
+// and most of a field's weight lies near its middle, while a ray's samples may
+// reach far beyond it (a four-level cascade: with the middle of the samples as
+// the base the error against binary64 was up to 1.7 times as large).
+__device__ __forceinline__ float base_param(const unsigned char* smem, const FieldLayout& L, int G,
+                                            const float o[3], const float d[3], float ta, float tb) {
+  const float4 m = *reinterpret_cast<const float4*>(smem + L.col + ((uint32_t)G + 1u) * sizeof(float4));
+  const float w = fmaf(m.x - o[0], d[0], fmaf(m.y - o[1], d[1], (m.z - o[2]) * d[2]));
+  const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
+  return fminf(fmaxf(__fdividef(w, dd), fminf(ta, tb)), fmaxf(ta, tb));
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -182,8 +210,8 @@ __device__ __forceinline__ void acc_clear(RayAcc& a) {
   a.r = a.g = a.b = splat(0.f);
 }
 
-// Fills the RayRec of one ray (one lane per ray): tb is any parameter, best
-// near the middle of the ray's samples.
+// Fills the RayRec of one ray (one lane per ray): tb is any parameter
+// (base_param).
 __device__ __forceinline__ void make_ray_rec(RayRec* rr, float2* len, const float o[3],
                                              const float d[3], float tb) {
   if (!(fabsf(tb) < 1e30f)) tb = 0.f;

@@ -103,14 +103,14 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
   if (nr > 0) {
     const uint32_t ka = sr[lane * kRunStride].x, kb = sr[lane * kRunStride + nr - 1].y;
     if (nr_all > kMaxRuns) my_next = (int)kb;
-    const float tb = 0.5f * (__ldg(lat.t + ka) + __ldg(lat.t + kb));
+    const float ta = __ldg(lat.t + ka), te = __ldg(lat.t + kb);
     float o[3], d[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, tb);
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, base_param(smem, L, G, o, d, ta, te));
     my_w = number_runs(sr + lane * kRunStride, nr);
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);

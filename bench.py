@@ -50,21 +50,23 @@ L2_FLUSH_BYTES = 256 << 20
 COMPOSITE_FP32_PER_BLOB = 6
 KERNELS_PER_TIMER = {"build_vdb": 4}   # the builder's timer spans four kernels
 # L2 hit rate and warp execution efficiency (active lanes per warp instruction) per kernel
-# from the ncu --set full captures (object frame, camera 0; unbounded: its first 200 image
+# from the ncu captures (object frame, camera 0; unbounded: its first 200 image
 # rows); dropped like the traffic when a kernel changes.
 PROFILED_COUNTERS = {
-    "object": {"hdda_walk": {"l2_hit_pct": 53.8, "active_lanes_of_32": 26.06},
-               "hdda_emit": {"l2_hit_pct": 10.7, "active_lanes_of_32": 27.16}},
-    "unbounded": {"hdda_walk": {"l2_hit_pct": 56.7, "active_lanes_of_32": 26.01},
-                  "hdda_emit": {"l2_hit_pct": 10.0, "active_lanes_of_32": 30.15}},
+    "object": {"hdda_walk": {"l2_hit_pct": 53.7, "active_lanes_of_32": 27.79},
+               "hdda_emit": {"l2_hit_pct": 10.7, "active_lanes_of_32": 27.18},
+               "composite": {"l2_hit_pct": 46.9, "active_lanes_of_32": 29.53}},
+    "unbounded": {"hdda_walk": {"l2_hit_pct": 57.5, "active_lanes_of_32": 26.28},
+                  "hdda_emit": {"l2_hit_pct": 10.0, "active_lanes_of_32": 30.15},
+                  "composite": {"l2_hit_pct": 38.6, "active_lanes_of_32": 29.96}},
 }
 # DRAM bytes (read + write) per launch from ncu of a workload's step on camera 0 (the
 # capture commands are kept with the profile summaries), for the roofline's "traffic"; an
 # entry must be dropped whenever its kernel changes, and a workload without a capture
 # reports none.
 PROFILED_TRAFFIC = {
-    "object": {"hdda_emit": 266_574_592, "hdda_walk": 16_295_424},
-    "unbounded": {"hdda_emit": 2_182_214_144, "hdda_walk": 27_365_888},
+    "object": {"hdda_emit": 269_658_880, "hdda_walk": 16_226_048, "composite": 226_914_304},
+    "unbounded": {"hdda_emit": 2_182_256_640, "hdda_walk": 33_935_616, "composite": 1_502_339_072},
 }
 
 

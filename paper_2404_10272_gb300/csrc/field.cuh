@@ -38,8 +38,8 @@
 // memory).  36 % of the instructions are the blob loop, the rest is per chunk
 // (listing, range, opacities, scan) and per ray (records).  Against two samples per lane of
 // whichever rays come next, with distances in space and colours scanned per
-// chunk, the compositor went from 434 to 292 us on an 800 x 800 object frame
-// and from 2367 to 1455 us on a 1245 x 825 unbounded one.  Tried: four lanes per ray
+// chunk, the compositor went from 434 to 297 us on an 800 x 800 object frame
+// and from 2367 to 1460 us on a 1245 x 825 unbounded one.  Tried: four lanes per ray
 // with eight samples each (a quarter fewer instructions, but 14 warps per SM:
 // 20 % slower), 16 lanes' worth of registers saved by loading behind the blob
 // loop (12 % slower), 7 CTAs per SM (spills, 15 % slower), CTAs of 8 to 16
@@ -95,7 +95,8 @@ struct RayRec {
 // would leave too few warps on an SM that way (eight at 256 blobs); there a
 // group has room for 5/8 of them, and a ray within reach of more takes each
 // chunk in passes (FieldWarp::more, kMany).  An 800 x 800 object frame takes
-// 0.62 -> 0.48 ms at 128 blobs and 1.62 -> 1.29 ms at 256 by this.
+// 0.62 -> 0.48 ms at 128 blobs and 1.62 -> 1.29 ms at 256 by this (0.45 and 1.22
+// since).
 constexpr int kAllBlobs = 64;
 
 struct FieldLayout {

@@ -1084,9 +1084,9 @@ int launch_walk(const WalkArgs& w, size_t smem, cudaStream_t s) {
   HDDA_CUDA_TRY(cudaGetDevice(&dev));
   // one resident wave, but no more CTAs than one per eight 32-ray tiles: a small call
   // is still spread over several SMs (its warps take tiles from the shared counter)
-  // without every SM staging the tables for warps that find no tile.  On the 96x96
-  // frame (288 tiles) the walk takes 0.0745 ms this way, 0.0792 ms with a CTA per
-  // tile and 0.0851 ms with a CTA per 32 tiles.
+  // without every SM staging the tables for warps that find no tile (30 us on the
+  // 96x96 frame, 288 tiles; one CTA per tile or per 32 tiles was 6 and 14 % slower
+  // when the walk took 75 us).
   const int64_t want = ((w.n + 31) / 32 + 7) / 8;
   const int64_t full = sm_count(dev);  // one CTA of 1024 fits (57 registers a thread)
   const unsigned grid = (unsigned)(want < full ? want : full);

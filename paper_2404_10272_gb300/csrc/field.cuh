@@ -48,8 +48,9 @@
 //
 // Rounding.  Ray parameters are taken relative to a base parameter near the
 // blobs (base_param), where the base point is rounded once, so t* and p carry
-// the rounding of coordinates near the blobs, not of the origin's.  Every product-sum is an explicit fused multiply-add, so the
-// arithmetic does not depend on the translation unit's contraction flags.
+// the rounding of coordinates near the blobs, not of the origin's.  Every
+// product-sum is an explicit fused multiply-add, so the arithmetic does not
+// depend on the translation unit's contraction flags.
 #pragma once
 
 #include <cmath>
@@ -86,7 +87,8 @@ struct RayRec {
 
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
 // tasks of R rays per warp: the blobs in pairs; [G + 1] colours (the last one black,
-// for padding) and the mean of the blobs' centres; then per warp [R] RayRec, [R] float2 and, per group, room for `cap`
+// for padding) and the mean of the blobs' centres; then per warp [R] RayRec,
+// [R] float2 and, per group, room for `cap`
 // records {k / 2, b = -k t*, c p^2 - log2 a, half-width | blob index} (and an
 // empty one behind them, for padding), as many list entries {offset of a
 // record, offset of its colour}, and `ring` factors of a faint ray.
@@ -168,8 +170,9 @@ __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayo
 // reach far beyond it (a four-level cascade: with the middle of the samples as
 // the base the error against binary64 was up to 1.7 times as large).
 __device__ __forceinline__ float base_param(const unsigned char* smem, const FieldLayout& L, int G,
-                                            const float o[3], const float d[3], float ta, float tb) {
-  const float4 m = *reinterpret_cast<const float4*>(smem + L.col + ((uint32_t)G + 1u) * sizeof(float4));
+                                            const float o[3], const float d[3], float ta,
+                                            float tb) {
+  const float4 m = reinterpret_cast<const float4*>(smem + L.col)[G + 1];
   const float w = fmaf(m.x - o[0], d[0], fmaf(m.y - o[1], d[1], (m.z - o[2]) * d[2]));
   const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
   return fminf(fmaxf(__fdividef(w, dd), fminf(ta, tb)), fmaxf(ta, tb));
@@ -555,7 +558,8 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
   const int task = __shfl_sync(kFieldFull, my_beg, ray & ~(kFaintRays - 1));
   const int gl = threadIdx.x & (kGroupLanes - 1);
   if (on)
-    *reinterpret_cast<float4*>(ring + (unsigned)q % kRing) = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+    *reinterpret_cast<float4*>(ring + (unsigned)q % kRing) =
+        make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
   __syncwarp();
   const int base = q - kPerLane * gl;  // the chunk's positions
   const int to = min(base + kChunk, end);

@@ -644,7 +644,8 @@ int launch_walk_emit_mode(const WalkArgs& w, size_t stage, bool skip, unsigned l
                           unsigned* emit_counter, int64_t* offsets, int32_t* ray_idx, float* t0,
                           float* t1, int64_t capacity, bool vec, int64_t* total,
                           cudaStream_t s) {
-  const bool sm = stage <= kMaxStageBytes;
+  // the record lists (131,328 bytes) take their share first: 101,120 bytes are left for the tables
+  const bool sm = walk_emit_smem(stage) <= kMaxCtaSmem;
   if (skip)
     return sm ? launch_walk_emit<kMode, true, true>(w, stage, state, emit_counter, offsets,
                                                    ray_idx, t0, t1, capacity, vec, total, s)

@@ -891,6 +891,7 @@ __host__ __device__ inline StageLayout stage_layout(int K, int L, int R, int64_t
 
 // leaves the L1 half of the SM's 256 KB
 constexpr size_t kMaxStageBytes = 128 * 1024;
+constexpr size_t kMaxCtaSmem = 227 * 1024;  // what one CTA can have on sm_103a
 
 template <typename T>
 __device__ __forceinline__ void stage_copy(T* dst, const T* __restrict__ src, int64_t count) {

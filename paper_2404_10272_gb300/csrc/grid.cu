@@ -788,8 +788,7 @@ int update_vdb(hdda_grid* g, const uint8_t* dense, const int64_t* blocks, int64_
     e = cudaMemcpyAsync(hw, flags + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) st = cuda_error(e, "cudaMemcpyAsync(status)");
   }
-  e = cudaFreeAsync(scratch, s);
-  if (st == HDDA_OK && e != cudaSuccess) st = cuda_error(e, "cudaFreeAsync");
+  st = scratch_free(scratch, s, st);
   if (st != HDDA_OK) return st;
   HDDA_CUDA_TRY(cudaEventRecord(g->built, s));
   if (dev_status) return HDDA_OK;

@@ -147,6 +147,9 @@ template <typename T>
 cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t s) {
   return scratch_alloc(reinterpret_cast<void**>(p), bytes, s);
 }
+// Gives a call's scratch back; returns the call's status `st`, or, if that was good, this
+// step's.
+int scratch_free(void* p, cudaStream_t s, int st);
 // A grid or batch came to life (+1) or was freed (-1) on a device: with the last
 // one the pool's unused memory is given back (runtime.cu).
 void scratch_users(int device, int change);

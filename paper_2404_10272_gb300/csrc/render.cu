@@ -476,8 +476,7 @@ extern "C" int hdda_render(const float* rays_o, const float* rays_d, int64_t n_r
     cudaError_t e = cudaMemcpyAsync(hw, scratch + 4, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) st = cuda_error(e, "cudaMemcpyAsync(status)");
   }
-  cudaError_t e = cudaFreeAsync(scratch, s);
-  if (st == HDDA_OK && e != cudaSuccess) st = cuda_error(e, "cudaFreeAsync");
+  st = scratch_free(scratch, s, st);
   if (st != HDDA_OK || dev_status) return st;
   HDDA_CUDA_TRY(cudaStreamSynchronize(s));
   if (*hw & kDevInternal) return set_error(HDDA_ERR_INTERNAL, "region check failed on the device");
@@ -528,7 +527,5 @@ extern "C" int hdda_traverse_composite(const float* rays_o, const float* rays_d,
   st = launch_sample_composite(rays_o, rays_d, n_rays, grid, lat, params->image_width, field,
                                n_gauss, rgba_out, offsets, ray_idx, t0, t1, capacity, dev_status,
                                scratch, s);
-  cudaError_t e = cudaFreeAsync(scratch, s);
-  if (st == HDDA_OK && e != cudaSuccess) st = cuda_error(e, "cudaFreeAsync");
-  return st;
+  return scratch_free(scratch, s, st);
 }

@@ -22,6 +22,7 @@ int set_error(int code, const char* fmt, ...) {
 }
 
 int cuda_error(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: the next call's launch checks must not find it again
   int code = (e == cudaErrorMemoryAllocation) ? HDDA_ERR_OOM : HDDA_ERR_CUDA;
   return set_error(code, "%s failed: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
@@ -82,6 +83,14 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
   e = pool_of(dev, &pool);
   if (e != cudaSuccess) return e;
   return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+int scratch_free(void* p, cudaStream_t s, int st) {
+  const cudaError_t e = cudaFreeAsync(p, s);
+  if (e == cudaSuccess) return st;
+  if (st == HDDA_OK) return cuda_error(e, "cudaFreeAsync");
+  cudaGetLastError();  // the call has reported its first error
+  return st;
 }
 
 void scratch_users(int device, int change) {

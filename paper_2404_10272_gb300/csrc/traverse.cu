@@ -969,9 +969,7 @@ int traverse(bool vdb, const float* ro, const float* rd, int64_t n, const hdda_g
   HDDA_CUDA_TRY(scratch_alloc(&scratch, twopass_scratch_bytes(n), s));
   st = run_twopass(ro, rd, n, grid, lat, params->image_width, offsets, ray_idx, t0, t1, capacity,
                    total_out, scratch, hw, nullptr, s);
-  cudaError_t e = cudaFreeAsync(scratch, s);
-  if (st == HDDA_OK && e != cudaSuccess) st = cuda_error(e, "cudaFreeAsync");
-  return st;
+  return scratch_free(scratch, s, st);
 }
 
 // The same two passes in stream order: no read-back and no synchronisation;
@@ -999,9 +997,7 @@ int traverse_async(const float* ro, const float* rd, int64_t n, const hdda_grid*
   HDDA_CUDA_TRY(scratch_alloc(&scratch, twopass_scratch_bytes(n), s));
   st = run_twopass(ro, rd, n, grid, lat, params->image_width, offsets, ray_idx, t0, t1,
                    capacity, &unused_total, scratch, nullptr, dev_status, s);
-  cudaError_t e = cudaFreeAsync(scratch, s);
-  if (st == HDDA_OK && e != cudaSuccess) st = cuda_error(e, "cudaFreeAsync");
-  return st;
+  return scratch_free(scratch, s, st);
 }
 
 }  // namespace

@@ -142,17 +142,17 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned)(min(q, end) - max(q - kChunk, beg));
+    RayLen* const rl = fw.lens(L) + max(ray, 0);
     float2 f[kPairs];
-    shade_chunk(sums, dt, acc, f);
-    float* const keep = &fw.lens(L)[max(ray, 0)].x;  // free once the ray's records are set up
-    if constexpr (!kMany)
-      faint_chunk(reinterpret_cast<float*>(smem + fw.recs + L.ring), keep, f, ray, q - kChunk, beg,
-                  end, my_beg, acc.T);
+    if (shade_chunk(sums, dt, ray, acc, f)) {  // uniform
+      if constexpr (kMany) acc.T *= faint_product(f);
+      else
+        faint_chunk(reinterpret_cast<float*>(smem + fw.recs + L.ring), rl, f, ray, q - kChunk, beg,
+                    end, my_beg, acc.S);
+    }
     const bool done = ray >= 0 && q - kPerLane * gl >= end;
     if (__any_sync(kFieldFull, done)) {
-      float T = acc.T;
-      if (!kMany && done && T > kFaint) T = *keep;
-      finish_rays(acc, T, done, rgba + 4 * ray);
+      finish_rays(acc, kMany ? acc.T : rl->T, done, rgba + 4 * ray);
       if (done) {
         ray = -1;
         beg = end = 0;

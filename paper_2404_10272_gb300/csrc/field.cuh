@@ -22,7 +22,7 @@
 // Rays never share a chunk, hence one record per blob and chunk serves all
 // of a group's samples, a 32-sample stretch of one ray meets few blobs it
 // does not need, the colour sums stay in registers until the ray ends, and a
-// scan over eight lanes (three steps) turns the samples' 1 - alpha into
+// scan over eight lanes (three steps) turns the samples' optical depths into
 // transmittances.
 //
 // Blob culling, in two stages.  setup_ray keeps the blobs within reach
@@ -79,16 +79,22 @@ __host__ __device__ inline int field_pairs(int G) { return (G + 63) / 64 * 32; }
 constexpr uint32_t kPairBytes = 3 * sizeof(float4) + sizeof(float2);
 
 // A ray as setup_ray reads it: base point and base parameter, direction and
-// 1 / |d|^2; beside it {|d|, the rounding margin of distances to its line}.
+// 1 / |d|^2; beside it a RayLen.
 struct RayRec {
   float4 base;  // o + tb d, tb
   float4 dir;   // d, 1 / |d|^2
 };
 
+// What else a ray keeps: |d|, the rounding margin of distances to its line, and the
+// transmittance of a faint ray (faint_chunk).
+struct RayLen {
+  float len, margin, T, unused;
+};
+
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
 // tasks of R rays per warp: the blobs in pairs; [G + 1] colours (the last one black,
 // for padding) and the mean of the blobs' centres; then per warp [R] RayRec,
-// [R] float2 and, per group, room for `cap`
+// [R] RayLen and, per group, room for `cap`
 // records {k / 2, b = -k t*, c p^2 - log2 a, half-width | blob index} (and an
 // empty one behind them, for padding), as many list entries {offset of a
 // record, offset of its colour}, and `ring` factors of a faint ray.
@@ -113,7 +119,7 @@ __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int
   L.col = (uint32_t)field_pairs(G) * kPairBytes;
   L.warp0 = L.col + ((uint32_t)G + 2u) * sizeof(float4);
   L.len = (uint32_t)R * sizeof(RayRec);
-  L.recs = L.len + (uint32_t)R * sizeof(float2);  // R is a multiple of 4
+  L.recs = L.len + (uint32_t)R * sizeof(RayLen);
   L.list = ((uint32_t)L.cap + 1u) * sizeof(float4);
   L.ring = L.list + (((uint32_t)L.cap + 1u) & ~1u) * sizeof(uint2);  // lists are padded to even
   L.group = L.ring + (uint32_t)ring * sizeof(float);
@@ -205,18 +211,20 @@ __device__ __forceinline__ float2 opacity_series2(float2 tau) {
 // One group's ray in work (the same values on the group's lanes except the
 // lane's colour sums).
 struct RayAcc {
-  float T;            // transmittance so far
+  float S;            // optical depth so far, times log2(e)
+  float T;            // faint ray: transmittance so far (faint_product)
   float2 r, g, b;     // this lane's colour sums (two halves, added at the end)
 };
 
 __device__ __forceinline__ void acc_clear(RayAcc& a) {
+  a.S = 0.f;
   a.T = 1.f;
   a.r = a.g = a.b = splat(0.f);
 }
 
 // Fills the RayRec of one ray (one lane per ray): tb is any parameter
 // (base_param).
-__device__ __forceinline__ void make_ray_rec(RayRec* rr, float2* len, const float o[3],
+__device__ __forceinline__ void make_ray_rec(RayRec* rr, RayLen* len, const float o[3],
                                              const float d[3], float tb) {
   if (!(fabsf(tb) < 1e30f)) tb = 0.f;
   float b[3];
@@ -231,7 +239,7 @@ __device__ __forceinline__ void make_ray_rec(RayRec* rr, float2* len, const floa
   const bool moves = dd > 1e-30f;
   rr->base = make_float4(b[0], b[1], b[2], tb);
   rr->dir = make_float4(d[0], d[1], d[2], moves ? 1.f / dd : 0.f);
-  *len = make_float2(moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm));
+  *len = RayLen{moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm), 1.f, 0.f};
 }
 
 // sqrt(x), approximately, rounded up and its low 8 bits replaced by a blob's
@@ -256,10 +264,11 @@ __device__ __forceinline__ float half_width(float x, int q) {
 // unbounded one and 1907 on a 1080p render-only one; two take 292, 1455, 1819.
 template <bool kMany>
 __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const RayRec* rr,
-                                         float2 len, float4* rec, int cap, int& q0) {
+                                         const RayLen* rl, float4* rec, int cap, int& q0) {
   const float4* tab = reinterpret_cast<const float4*>(smem);
   const int lane = threadIdx.x & 31, np = field_pairs(G);
   const float4 B = rr->base, D = rr->dir;
+  const float2 len = *reinterpret_cast<const float2*>(rl);  // |d|, margin
   const float2 dx = splat(D.x), dy = splat(D.y), dz = splat(D.z), nw = splat(-D.w);
   int n = 0;
   for (; q0 < G; q0 += 64) {
@@ -273,7 +282,6 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     float2 ts = __fmul2_rn(nw, __ffma2_rn(wx, dx, __ffma2_rn(wy, dy, __fmul2_rn(wz, dz))));
     float2 qx = __ffma2_rn(ts, dx, wx), qy = __ffma2_rn(ts, dy, wy), qz = __ffma2_rn(ts, dz, wz);
     const float2 de = __fmul2_rn(nw, __ffma2_rn(qx, dx, __ffma2_rn(qy, dy, __fmul2_rn(qz, dz))));
-    ts = __fadd2_rn(ts, de);
     qx = __ffma2_rn(de, dx, qx);
     qy = __ffma2_rn(de, dy, qy);
     qz = __ffma2_rn(de, dz, qz);
@@ -281,7 +289,8 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     const float2 hl = __ffma2_rn(rc, splat(len.y), reach);
     const float2 lim2 = __ffma2_rn(hl, hl, make_float2(-cp2.x, -cp2.y));
     const float2 k = __fmul2_rn(rc, splat(len.x));
-    const float2 hk = __fmul2_rn(splat(0.5f), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
+    const float2 hk = __fmul2_rn(splat(0.5f), k), nk = make_float2(-k.x, -k.y);
+    const float2 b = __ffma2_rn(nk, ts, __fmul2_rn(nk, de));  // -k (ts + de), rounded once
     const float2 e = __fadd2_rn(cp2, make_float2(-AK.x, -AK.y));
     const int q = q0 + lane;
     const bool near0 = lim2.x >= 0.f && q < G, near1 = lim2.y >= 0.f && q + 32 < G;
@@ -347,8 +356,8 @@ struct FieldWarp {
     return reinterpret_cast<RayRec*>(smem + rays_at(L));
   }
 
-  __device__ __forceinline__ float2* lens(const FieldLayout& L) const {
-    return reinterpret_cast<float2*>(smem + rays_at(L) + L.len);
+  __device__ __forceinline__ RayLen* lens(const FieldLayout& L) const {
+    return reinterpret_cast<RayLen*>(smem + rays_at(L) + L.len);
   }
 
   __device__ __forceinline__ void init(unsigned char* smem_, const FieldLayout& L) {
@@ -372,7 +381,7 @@ struct FieldWarp {
   // The records of group g for ray i of the task, from blob q0 on.
   __device__ __forceinline__ void setup(const FieldLayout& L, int G, int g, int i, int q0 = 0) {
     const uint32_t rec = rays_at(L) + L.recs + (uint32_t)g * L.group;
-    const int m = setup_ray<kMany>(smem, G, rays(L) + i, lens(L)[i],
+    const int m = setup_ray<kMany>(smem, G, rays(L) + i, lens(L) + i,
                                    reinterpret_cast<float4*>(smem + rec), L.cap, q0);
     if ((int)(threadIdx.x & 31) / kGroupLanes == g) {
       nc = m;
@@ -461,100 +470,123 @@ __device__ __forceinline__ void sums_clear(BlobSums& S) {
   for (int h = 0; h < kPairs; ++h) S.s[h] = S.r[h] = S.g[h] = S.b[h] = splat(0.f);
 }
 
+// The limit, in optical depth times log2(e), below which a ray is faint: its
+// transmittance is above 0.98.
+//
+// A ray's transmittance comes from the sum of its optical depths, chunk by
+// chunk: a product of (1 - alpha) rounds every factor to a multiple of 6e-8 and
+// every product again.  Error against binary64 (2-norm, relative) as a product
+// and as a sum: 1.9e-7 and 1.1e-7 on object frames, 6.1e-7 and 2.7e-7 on
+// unbounded ones.  Only the lane's own four samples are a product: with an
+// exponential for each, the compositor was 7 % slower for the same error.
+// A faint ray's opacity is the exception: it is taken as 1 minus a product of
+// (1 - alpha) in a fixed order, that of faint_chunk for stored samples and up
+// to kAllBlobs blobs, else that of faint_product, chunk after chunk.  The roundings above are
+// 2e-4 of so small an opacity, and callers may compare frames with stored ones
+// by their values: so its roundings stay what they were.
+constexpr float kFaintDepth = 0.029146346f;  // -log2(0.98)
+
 // Accumulates a chunk's samples of lengths dt = t1 - t0 (0 for padding) front
-// to back: multiplies into the group's transmittance and adds to the lane's
-// colour sums; f receives the samples' 1 - alpha.
-__device__ __forceinline__ void shade_chunk(BlobSums& B, const float2 dt[kPairs], RayAcc& acc,
-                                            float2 f[kPairs]) {
+// to back: adds to the group's optical depth and to the lane's colour sums.
+// f receives the samples' 1 - alpha.  Returns whether some group's ray (`ray` >=
+// 0) is still faint.
+__device__ __forceinline__ bool shade_chunk(BlobSums& B, const float2 dt[kPairs], int ray,
+                                            RayAcc& acc, float2 f[kPairs]) {
   const int gl = threadIdx.x & (kGroupLanes - 1);
-  float2(&sig)[kPairs] = B.s;
+  float2(&tau)[kPairs] = B.s;  // densities, now optical depths
   const float2(&cr)[kPairs] = B.r, (&cg)[kPairs] = B.g, (&cb)[kPairs] = B.b;
-  // optical depths (sig becomes tau), opacities, and the opacity per density
+#pragma unroll
+  for (int h = 0; h < kPairs; ++h) tau[h] = __fmul2_rn(tau[h], dt[h]);
+  // depth before the lane's first sample: the ray's so far, the lanes before
+  float inc = kLog2e * ((tau[0].x + tau[0].y) + (tau[1].x + tau[1].y));
+#pragma unroll
+  for (int o = 1; o < kGroupLanes; o <<= 1) {
+    const float y = __shfl_up_sync(kFieldFull, inc, o, kGroupLanes);
+    if (gl >= o) inc += y;
+  }
+  float before = __shfl_up_sync(kFieldFull, inc, 1, kGroupLanes);
+  before = gl ? acc.S + before : acc.S;
+  acc.S += __shfl_sync(kFieldFull, inc, kGroupLanes - 1, kGroupLanes);
+  // opacities, and the opacity per density
   float2 al[kPairs], op[kPairs];
   float tm = 0.f;
 #pragma unroll
   for (int h = 0; h < kPairs; ++h) {
-    sig[h] = __fmul2_rn(sig[h], dt[h]);
-    const float2 p = opacity_series2(sig[h]);
-    al[h] = __fmul2_rn(sig[h], p);
+    const float2 p = opacity_series2(tau[h]);
+    al[h] = __fmul2_rn(tau[h], p);
     op[h] = __fmul2_rn(dt[h], p);
-    tm = fmaxf(tm, fmaxf(fabsf(sig[h].x), fabsf(sig[h].y)));
+    tm = fmaxf(tm, fmaxf(fabsf(tau[h].x), fabsf(tau[h].y)));
   }
   if (!(tm < 0.5f)) {  // 1 - exp2: its absolute error of a few 1e-8 is small against >= 0.39
 #pragma unroll
     for (int h = 0; h < kPairs; ++h) {
       // (1 - exp(-tau)) / sigma = (1 - exp(-tau)) dt / tau
-      if (!(fabsf(sig[h].x) < 0.5f)) {
-        al[h].x = 1.f - ex2_approx(-kLog2e * sig[h].x);
-        op[h].x = __fdividef(al[h].x * dt[h].x, sig[h].x);
+      if (!(fabsf(tau[h].x) < 0.5f)) {
+        al[h].x = 1.f - ex2_approx(-kLog2e * tau[h].x);
+        op[h].x = __fdividef(al[h].x * dt[h].x, tau[h].x);
       }
-      if (!(fabsf(sig[h].y) < 0.5f)) {
-        al[h].y = 1.f - ex2_approx(-kLog2e * sig[h].y);
-        op[h].y = __fdividef(al[h].y * dt[h].y, sig[h].y);
+      if (!(fabsf(tau[h].y) < 0.5f)) {
+        al[h].y = 1.f - ex2_approx(-kLog2e * tau[h].y);
+        op[h].y = __fdividef(al[h].y * dt[h].y, tau[h].y);
       }
     }
   }
-  // transmittance before each sample: the ray's so far, the lanes before, the
-  // lane's earlier samples
-  float run = 1.f;
-  float2 bef[kPairs];
+  // transmittance before each sample: of the depth before the lane, times the
+  // lane's earlier samples' 1 - alpha
+  float run = ex2_approx(-before);
 #pragma unroll
   for (int h = 0; h < kPairs; ++h) {
     f[h] = __ffma2_rn(al[h], splat(-1.f), splat(1.f));
-    bef[h].x = run;
-    run *= f[h].x;
-    bef[h].y = run;
-    run *= f[h].y;
-  }
-  float inc = run;
-#pragma unroll
-  for (int o = 1; o < kGroupLanes; o <<= 1) {
-    const float y = __shfl_up_sync(kFieldFull, inc, o, kGroupLanes);
-    if (gl >= o) inc *= y;
-  }
-  float before = __shfl_up_sync(kFieldFull, inc, 1, kGroupLanes);
-  before = gl ? acc.T * before : acc.T;
-  acc.T *= __shfl_sync(kFieldFull, inc, kGroupLanes - 1, kGroupLanes);
-#pragma unroll
-  for (int h = 0; h < kPairs; ++h) {
-    const float2 g = __fmul2_rn(op[h], __fmul2_rn(bef[h], splat(before)));
+    const float mid = run * f[h].x;
+    const float2 g = __fmul2_rn(op[h], make_float2(run, mid));
+    run = mid * f[h].y;
     acc.r = __ffma2_rn(g, cr[h], acc.r);
     acc.g = __ffma2_rn(g, cg[h], acc.g);
     acc.b = __ffma2_rn(g, cb[h], acc.b);
   }
+  return __any_sync(kFieldFull, ray >= 0 && acc.S < kFaintDepth);
 }
 
-// The transmittance of faint rays (stored samples, up to kAllBlobs blobs).  1 -
-// alpha is rounded to a multiple of 6e-8, and so is every product of such
-// factors near 1: where a ray is nearly transparent, the order of the
-// products shows in its pixel's opacity (2e-4 of it on a frame that faint).  A
-// ray whose transmittance stays above kFaint therefore takes it as a product
-// in a fixed order: of the samples of four rays (ray / 4), each 64 in a row are
-// a segment; a segment's samples of one ray are a balanced tree over the pairs
-// of places, counted back from the last whole pair, times a last single
-// sample; segments multiply in order.  Between chunks the factors wait in a
-// ring of 96 per group in shared memory.  It costs the compositor 3 to 5 %
-// (291 -> 304 us on the object frame, 1435 -> 1482 on the unbounded one before
-// setup_ray took two blobs per lane; 322 and 1571 with the product and `task` in
-// registers, which then spill).  The limit: with 0.998
-// three of 81 random unbounded frames differ by 2.1e-5 (2-norm, relative) from
-// the same product order throughout, with 0.98 none by more than 7.5e-6.
-constexpr float kFaint = 0.98f;
+// A finished ray's opacity, from its optical depth or, faint, its transmittance T.
+__device__ __forceinline__ float ray_opacity(float S, float T) {
+  return 1.f - (S < kFaintDepth ? T : ex2_approx(-S));
+}
+
+// A chunk's product for faint rays, called by the whole warp: the lane's four
+// factors in turn, then a tree over the group's lanes.
+__device__ __forceinline__ float faint_product(const float2 f[kPairs]) {
+  float m = f[0].x * f[0].y;
+#pragma unroll
+  for (int h = 1; h < kPairs; ++h) {
+    m *= f[h].x;
+    m *= f[h].y;
+  }
+#pragma unroll
+  for (int o = 1; o < kGroupLanes; o <<= 1) m *= __shfl_xor_sync(kFieldFull, m, o);
+  return m;
+}
+
+// The product for stored samples and up to kAllBlobs blobs: the samples of four
+// rays (ray / 4), each 64 in a row, are a segment; a segment's samples of one
+// ray are a balanced tree over the pairs of places, counted back from the last
+// whole pair, times a last single sample; segments multiply in order.  Between
+// chunks the factors wait in a ring of 96 per group in shared memory.  The
+// limit: with 0.998 three of 81 random unbounded frames differ by 2.1e-5
+// (2-norm, relative) from the same product order throughout, with 0.98 none by more
+// than 7.5e-6.
 constexpr int kFaintRays = 4;
 constexpr int kRing = 96;  // a segment and a chunk beyond it
 
-// One chunk of every group, called by the whole warp: `f` the lane's factors (1
-// for padding), `q` its first position (a multiple of 4), `busy` where the
-// group has ray `ray` (else -1) of positions [beg, end), `T` the ray's
-// transmittance behind the chunk; lane i's `my_beg` is the first position of
-// ray i.  The product so far stays in *keep (as `task`, it takes no register
-// of the blob loop's).
-__device__ __forceinline__ void faint_chunk(float* ring, float* keep, const float2 f[kPairs],
+// One chunk of every group, called by the whole warp when some ray is faint: `f`
+// the lane's factors (1 for padding), `q` its first position (a multiple of 4),
+// `ray` the group's ray (-1: none) of positions [beg, end), `S` its depth
+// behind the chunk; lane i's `my_beg` is the first position of ray i.  The
+// product so far stays in rl->T (it takes no register of the blob loop's).
+__device__ __forceinline__ void faint_chunk(float* ring, RayLen* rl, const float2 f[kPairs],
                                             int ray, int q, int beg, int end, int my_beg,
-                                            float T) {
+                                            float S) {
   static_assert(kPairs == 2, "one 16-byte store per lane");
-  const bool on = ray >= 0 && T > kFaint;
-  if (!__any_sync(kFieldFull, on)) return;
+  const bool on = ray >= 0 && S < kFaintDepth;
   const int task = __shfl_sync(kFieldFull, my_beg, ray & ~(kFaintRays - 1));
   const int gl = threadIdx.x & (kGroupLanes - 1);
   if (on)
@@ -564,8 +596,7 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
   const int base = q - kPerLane * gl;  // the chunk's positions
   const int to = min(base + kChunk, end);
   int at = max(beg, base);  // a position of the segment in work
-  float F = 1.f;
-  if (on && base > beg) F = *keep;
+  float F = rl->T;
   __syncwarp();
 #pragma unroll 1
   for (int turn = 0; turn < 2; ++turn) {  // a chunk ends two segments at most
@@ -593,7 +624,7 @@ __device__ __forceinline__ void faint_chunk(float* ring, float* keep, const floa
       at = s1;  // on to the next segment
     }
   }
-  if (on) *keep = F;  // the same value from the group's lanes
+  if (on) rl->T = F;  // the same value from the group's lanes
   __syncwarp();       // the ring may be overwritten
 }
 
@@ -643,7 +674,7 @@ __device__ __forceinline__ void chunk_params(const float2 a[kPairs], const float
 // Writes the pixels of the groups whose ray is done (called by the whole
 // warp): the colour sums are added up over the group's eight lanes, each pair
 // of lanes ending with one channel.
-// `T` is the transmittance of the whole ray.
+// `T` is the transmittance of a faint ray.
 __device__ __forceinline__ void finish_rays(const RayAcc& acc, float T, bool done, float* px) {
   static_assert(kGroupLanes == 8, "two lanes per channel");
   const int gl = threadIdx.x & (kGroupLanes - 1);
@@ -654,7 +685,7 @@ __device__ __forceinline__ void finish_rays(const RayAcc& acc, float T, bool don
   const float v = (up ? 0.f : g) + __shfl_xor_sync(kFieldFull, up ? g : 0.f, 4);
   u = (odd ? v : u) + __shfl_xor_sync(kFieldFull, odd ? u : v, 2);
   u += __shfl_xor_sync(kFieldFull, u, 1);
-  if (gl == 6) u = 1.f - T;
+  if (gl == 6) u = ray_opacity(acc.S, T);
   if (done && !(gl & 1)) px[gl >> 1] = u;
 }
 

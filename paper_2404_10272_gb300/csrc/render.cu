@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned) min(kChunk, W - q);
     float2 f[kPairs];
-    shade_chunk(sums, dt, acc, f);
+    if (shade_chunk(sums, dt, ray, acc, f)) acc.T *= faint_product(f);  // uniform
     q += kChunk;
     const bool round_over = ray >= 0 && q - kPerLane * gl >= W;
     bool done = round_over && k_next >= lat.K;

@@ -282,6 +282,7 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     float2 ts = __fmul2_rn(nw, __ffma2_rn(wx, dx, __ffma2_rn(wy, dy, __fmul2_rn(wz, dz))));
     float2 qx = __ffma2_rn(ts, dx, wx), qy = __ffma2_rn(ts, dy, wy), qz = __ffma2_rn(ts, dz, wz);
     const float2 de = __fmul2_rn(nw, __ffma2_rn(qx, dx, __ffma2_rn(qy, dy, __fmul2_rn(qz, dz))));
+    ts = __fadd2_rn(ts, de);
     qx = __ffma2_rn(de, dx, qx);
     qy = __ffma2_rn(de, dy, qy);
     qz = __ffma2_rn(de, dz, qz);
@@ -289,8 +290,7 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     const float2 hl = __ffma2_rn(rc, splat(len.y), reach);
     const float2 lim2 = __ffma2_rn(hl, hl, make_float2(-cp2.x, -cp2.y));
     const float2 k = __fmul2_rn(rc, splat(len.x));
-    const float2 hk = __fmul2_rn(splat(0.5f), k), nk = make_float2(-k.x, -k.y);
-    const float2 b = __ffma2_rn(nk, ts, __fmul2_rn(nk, de));  // -k (ts + de), rounded once
+    const float2 hk = __fmul2_rn(splat(0.5f), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
     const float2 e = __fadd2_rn(cp2, make_float2(-AK.x, -AK.y));
     const int q = q0 + lane;
     const bool near0 = lim2.x >= 0.f && q < G, near1 = lim2.y >= 0.f && q + 32 < G;

@@ -54,21 +54,21 @@ __device__ __forceinline__ void load_lane(const float* __restrict__ t0, const fl
   }
 }
 
-template <bool kVec, bool kMany>
+template <bool kVec, int kForm>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R,
     const int64_t* __restrict__ offsets, const float* __restrict__ t0,
     const float* __restrict__ t1, const float* __restrict__ field, int G,
     float* __restrict__ rgba, bool count_evals) {
   extern __shared__ __align__(16) unsigned char smem[];  // field_layout
-  const FieldLayout L = field_layout(G, kWarpsPerCta, R, kMany ? 0 : kRing);
-  stage_blobs(smem, L, field, G);
+  const FieldLayout L = field_layout(G, kWarpsPerCta, R, kForm == kMany ? 0 : kRing);
+  stage_blobs<kForm>(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int grp = lane / kGroupLanes, gl = lane & (kGroupLanes - 1);
   const int64_t first = ((int64_t)blockIdx.x * kWarpsPerCta + wib) * R;
   if (first >= n) return;  // uniform per warp; no block barrier follows
-  FieldWarp<kMany> fw;
+  FieldWarp<kForm> fw;
   fw.init(smem, L);
 
   // lane i < R holds ray i's range, relative to the warp's first position
@@ -112,6 +112,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     unsigned idle = __ballot_sync(kFieldFull, ray < 0) & kLeaders;  // groups without a ray
     if (idle) {  // uniform
       if (!pending && idle == kLeaders) break;
+      const bool was_idle = ray < 0;
       while (idle && pending) {
         const int g = (__ffs(idle) - 1) / kGroupLanes, i = __ffs(pending) - 1;
         idle &= idle - 1;
@@ -125,8 +126,9 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
           load_lane<kVec>(t0, t1, q, beg, end, lim, a, b);
           tb = fw.rays(L)[i].base.w;
         }
-        fw.setup(L, G, g, i);
+        if constexpr (kForm != kFew) fw.setup(L, G, g, i);
       }
+      if constexpr (kForm == kFew) fw.setup_own(L, G, was_idle && ray >= 0, ray);
       fw.ready();
     }
     float2 t[kPairs], dt[kPairs];
@@ -139,20 +141,21 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     BlobSums sums;
     sums_clear(sums);
     sum_blobs(smem, fw.recs + L.list, len, t, sums);
-    if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
+    if constexpr (kForm == kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned)(min(q, end) - max(q - kChunk, beg));
     RayLen* const rl = fw.lens(L) + max(ray, 0);
     float2 f[kPairs];
-    if (shade_chunk(sums, dt, ray, acc, f)) {  // uniform
-      if constexpr (kMany) acc.T *= faint_product(f);
-      else
-        faint_chunk(reinterpret_cast<float*>(smem + fw.recs + L.ring), rl, f, ray, q - kChunk, beg,
-                    end, my_beg, acc.S);
+    const bool faint = shade_chunk(sums, dt, ray, acc, f);
+    if constexpr (kForm == kMany) {
+      faint_product(f, faint, acc);
+    } else if (__any_sync(kFieldFull, faint)) {
+      faint_chunk(reinterpret_cast<float*>(smem + fw.recs + L.ring), rl, f, faint, ray, q - kChunk,
+                  beg, end, my_beg, acc.S);
     }
     const bool done = ray >= 0 && q - kPerLane * gl >= end;
     if (__any_sync(kFieldFull, done)) {
-      finish_rays(acc, kMany ? acc.T : rl->T, done, rgba + 4 * ray);
+      finish_rays(acc, kForm == kMany ? acc.T : rl->T, done, rgba + 4 * ray);
       if (done) {
         ray = -1;
         beg = end = 0;
@@ -198,9 +201,11 @@ extern "C" int hdda_composite(const float* rays_o, const float* rays_d, int64_t 
   const unsigned grid = (unsigned)blocks;
   const FieldLayout L = field_layout(n_gauss, kWarpsPerCta, R, n_gauss <= kAllBlobs ? kRing : 0);
   const bool vec = ((reinterpret_cast<uintptr_t>(t0) | reinterpret_cast<uintptr_t>(t1)) & 15) == 0;
-  const auto kern = n_gauss <= kAllBlobs
-                        ? (vec ? composite_kernel<true, false> : composite_kernel<false, false>)
-                        : (vec ? composite_kernel<true, true> : composite_kernel<false, true>);
+  const auto kern = n_gauss <= kFewBlobs
+                        ? (vec ? composite_kernel<true, kFew> : composite_kernel<false, kFew>)
+                    : n_gauss <= kAllBlobs
+                        ? (vec ? composite_kernel<true, kSome> : composite_kernel<false, kSome>)
+                        : (vec ? composite_kernel<true, kMany> : composite_kernel<false, kMany>);
   if (L.bytes > 48 * 1024)
     HDDA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)L.bytes));

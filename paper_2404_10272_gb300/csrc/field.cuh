@@ -71,10 +71,11 @@ constexpr unsigned kLeaders = 0xffffffffu / ((1u << kGroupLanes) - 1u);  // the 
 constexpr int kChunk = kGroupLanes * kPerLane;       // samples of one ray per step
 constexpr float kLog2e = 1.4426950408889634f;
 
-// The blobs as setup_ray reads them, two per lane: pair p holds blobs b = (p /
-// 32) * 64 + p % 32 and b + 32 in four arrays over the pairs (16 bytes per lane
-// and load, consecutive lanes consecutive): {-mu_x, -mu_y}, {-mu_z, c}, {log2 a,
-// sqrt(c)} and sqrt(c) (kCullSigmas s + margin), each as both blobs' values.
+// The blobs as setup_ray reads them, two per lane, w lanes at a time (w = 32; 8 for
+// kFew): pair p holds blobs b = (p / w) * 2 w + p % w and b + w in four arrays over
+// the pairs (16 bytes per lane and load, consecutive lanes consecutive): {-mu_x,
+// -mu_y}, {-mu_z, c}, {log2 a, sqrt(c)} and sqrt(c) (kCullSigmas s + margin),
+// each as both blobs' values.
 __host__ __device__ inline int field_pairs(int G) { return (G + 63) / 64 * 32; }
 constexpr uint32_t kPairBytes = 3 * sizeof(float4) + sizeof(float2);
 
@@ -107,6 +108,11 @@ struct RayLen {
 // since).
 constexpr int kAllBlobs = 64;
 
+// Up to kFewBlobs blobs the compositor's groups each set up their own ray (kFew).
+constexpr int kFewBlobs = 32;
+
+enum FieldForm { kFew, kSome, kMany };
+
 struct FieldLayout {
   uint32_t col, warp0, per_warp, len, recs, list, ring, group, bytes;
   int cap;
@@ -130,6 +136,7 @@ __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int
 
 // Stages `G` blobs of 8 floats {mu[3], s, a, rgb[3]} (block-wide; the caller
 // synchronises the block afterwards).
+template <int kForm>
 __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayout& L,
                                             const float* __restrict__ field, int G) {
   float* tab = reinterpret_cast<float*>(smem);
@@ -140,7 +147,8 @@ __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayo
     const float s = f[3], c = kLog2e / (2.f * s * s), rc = sqrtf(c);
     const float reach = kCullSigmas * s;
     const float mu_max = fmaxf(fabsf(f[0]), fmaxf(fabsf(f[1]), fabsf(f[2])));
-    const int p = (i >> 6) * 32 + (i & 31), h = (i >> 5) & 1;  // the pair, its blob
+    constexpr int w = kForm == kFew ? kGroupLanes : 32;
+    const int p = i / (2 * w) * w + i % w, h = i / w & 1;  // the pair, its blob
     float *xy = tab + 4 * p + h, *zc = xy + 4 * np, *ak = zc + 4 * np;
     xy[0] = -f[0];
     xy[2] = -f[1];
@@ -262,16 +270,20 @@ __device__ __forceinline__ float half_width(float x, int q) {
 // vector, so their rounding is that of the distance, not of the span from the
 // base point.  A blob per lane took 304 us on the object frame, 1482 on the
 // unbounded one and 1907 on a 1080p render-only one; two take 292, 1455, 1819.
-template <bool kMany>
+// With kFew every group's eight lanes work on its own ray, where `on`.
+template <int kForm>
 __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const RayRec* rr,
-                                         const RayLen* rl, float4* rec, int cap, int& q0) {
+                                         const RayLen* rl, float4* rec, int cap, int& q0,
+                                         bool on = true) {
+  constexpr int w = kForm == kFew ? kGroupLanes : 32;  // lanes on the ray
   const float4* tab = reinterpret_cast<const float4*>(smem);
-  const int lane = threadIdx.x & 31, np = field_pairs(G);
+  const int lane = threadIdx.x & (w - 1), first = (threadIdx.x & 31) - lane, np = field_pairs(G);
+  const unsigned mine = (kFieldFull >> (32 - w)) << first;
   const float4 B = rr->base, D = rr->dir;
   const float2 len = *reinterpret_cast<const float2*>(rl);  // |d|, margin
   const float2 dx = splat(D.x), dy = splat(D.y), dz = splat(D.z), nw = splat(-D.w);
   int n = 0;
-  for (; q0 < G; q0 += 64) {
+  for (; q0 < G; q0 += 2 * w) {
     const int p = (q0 >> 1) + lane;
     const float4 XY = tab[p], ZC = tab[np + p], AK = tab[2 * np + p];
     const float2 reach = reinterpret_cast<const float2*>(tab + 3 * np)[p];
@@ -293,16 +305,16 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     const float2 hk = __fmul2_rn(splat(0.5f), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
     const float2 e = __fadd2_rn(cp2, make_float2(-AK.x, -AK.y));
     const int q = q0 + lane;
-    const bool near0 = lim2.x >= 0.f && q < G, near1 = lim2.y >= 0.f && q + 32 < G;
-    const unsigned ball0 = __ballot_sync(kFieldFull, near0);
-    const unsigned ball1 = __ballot_sync(kFieldFull, near1);
+    const bool near0 = on && lim2.x >= 0.f && q < G, near1 = on && lim2.y >= 0.f && q + w < G;
+    const unsigned ball0 = __ballot_sync(kFieldFull, near0) & mine;
+    const unsigned ball1 = __ballot_sync(kFieldFull, near1) & mine;
     const int n0 = __popc(ball0), kept = n0 + __popc(ball1);
-    if (kMany && n + kept > cap) break;  // uniform; one step always fits
-    const unsigned below = (1u << lane) - 1u;
+    if (kForm == kMany && n + kept > cap) break;  // uniform; one step always fits
+    const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
     if (near0)
       rec[n + __popc(ball0 & below)] = make_float4(hk.x, b.x, e.x, half_width(lim2.x, q));
     if (near1)
-      rec[n + n0 + __popc(ball1 & below)] = make_float4(hk.y, b.y, e.y, half_width(lim2.y, q + 32));
+      rec[n + n0 + __popc(ball1 & below)] = make_float4(hk.y, b.y, e.y, half_width(lim2.y, q + w));
     n += kept;
   }
   return n;
@@ -340,7 +352,7 @@ __device__ __forceinline__ void sum_blobs(const unsigned char* smem, uint32_t li
 
 // A warp's groups over one task: where their shared memory is, and each
 // group's blob records (the same values on the group's lanes).
-template <bool kMany>
+template <int kForm>
 struct FieldWarp {
   unsigned char* smem;
   uint32_t recs;  // the group's records
@@ -375,18 +387,30 @@ struct FieldWarp {
   // The group has no ray.
   __device__ __forceinline__ void release() {
     nc = 0;
-    if constexpr (kMany) next = kMaxGauss;
+    if constexpr (kForm == kMany) next = kMaxGauss;
   }
 
   // The records of group g for ray i of the task, from blob q0 on.
   __device__ __forceinline__ void setup(const FieldLayout& L, int G, int g, int i, int q0 = 0) {
     const uint32_t rec = rays_at(L) + L.recs + (uint32_t)g * L.group;
-    const int m = setup_ray<kMany>(smem, G, rays(L) + i, lens(L) + i,
+    const int m = setup_ray<kForm>(smem, G, rays(L) + i, lens(L) + i,
                                    reinterpret_cast<float4*>(smem + rec), L.cap, q0);
     if ((int)(threadIdx.x & 31) / kGroupLanes == g) {
       nc = m;
-      if constexpr (kMany) next = q0;
+      if constexpr (kForm == kMany) next = q0;
     }
+  }
+
+  // kFew: the records of every group whose ray, `ray` of the task, is new (`on`).
+  // Rays of a few samples often end together: 640,000 of two samples took 214 us
+  // over 16 blobs and 226 over 32 with the whole warp on one group after the
+  // other, 171 and 199 so (of 20 samples over 32 blobs 306 either way).
+  __device__ __forceinline__ void setup_own(const FieldLayout& L, int G, bool on, int ray) {
+    const int i = max(ray, 0);
+    int q0 = 0;
+    const int m = setup_ray<kForm>(smem, G, rays(L) + i, lens(L) + i,
+                                   reinterpret_cast<float4*>(smem + recs), L.cap, q0, on);
+    if (on) nc = m;
   }
 
   // After setups: they are visible, `most` is up to date.
@@ -485,10 +509,11 @@ __device__ __forceinline__ void sums_clear(BlobSums& S) {
 // 2e-4 of so small an opacity, and callers may compare frames with stored ones
 // by their values: so its roundings stay what they were.
 constexpr float kFaintDepth = 0.029146346f;  // -log2(0.98)
+constexpr float kNoDepth = 1.f / (1 << 26);  // below it every 1 - alpha of a ray is 1
 
 // Accumulates a chunk's samples of lengths dt = t1 - t0 (0 for padding) front
 // to back: adds to the group's optical depth and to the lane's colour sums.
-// f receives the samples' 1 - alpha.  Returns whether some group's ray (`ray` >=
+// f receives the samples' 1 - alpha.  Returns whether the group's ray (`ray` >=
 // 0) is still faint.
 __device__ __forceinline__ bool shade_chunk(BlobSums& B, const float2 dt[kPairs], int ray,
                                             RayAcc& acc, float2 f[kPairs]) {
@@ -544,7 +569,7 @@ __device__ __forceinline__ bool shade_chunk(BlobSums& B, const float2 dt[kPairs]
     acc.g = __ffma2_rn(g, cg[h], acc.g);
     acc.b = __ffma2_rn(g, cb[h], acc.b);
   }
-  return __any_sync(kFieldFull, ray >= 0 && acc.S < kFaintDepth);
+  return ray >= 0 && acc.S < kFaintDepth;
 }
 
 // A finished ray's opacity, from its optical depth or, faint, its transmittance T.
@@ -552,9 +577,11 @@ __device__ __forceinline__ float ray_opacity(float S, float T) {
   return 1.f - (S < kFaintDepth ? T : ex2_approx(-S));
 }
 
-// A chunk's product for faint rays, called by the whole warp: the lane's four
-// factors in turn, then a tree over the group's lanes.
-__device__ __forceinline__ float faint_product(const float2 f[kPairs]) {
+// The transmittance of faint rays (`faint` on the group's lanes) behind a chunk,
+// in the chunk's order: the lane's four factors in turn, then a tree over the
+// group's lanes.  Called by the whole warp.
+__device__ __forceinline__ void faint_product(const float2 f[kPairs], bool faint, RayAcc& acc) {
+  if (!__any_sync(kFieldFull, faint && !(fabsf(acc.S) < kNoDepth))) return;
   float m = f[0].x * f[0].y;
 #pragma unroll
   for (int h = 1; h < kPairs; ++h) {
@@ -563,7 +590,7 @@ __device__ __forceinline__ float faint_product(const float2 f[kPairs]) {
   }
 #pragma unroll
   for (int o = 1; o < kGroupLanes; o <<= 1) m *= __shfl_xor_sync(kFieldFull, m, o);
-  return m;
+  acc.T *= m;
 }
 
 // The product for stored samples and up to kAllBlobs blobs: the samples of four
@@ -577,21 +604,24 @@ __device__ __forceinline__ float faint_product(const float2 f[kPairs]) {
 constexpr int kFaintRays = 4;
 constexpr int kRing = 96;  // a segment and a chunk beyond it
 
-// One chunk of every group, called by the whole warp when some ray is faint: `f`
-// the lane's factors (1 for padding), `q` its first position (a multiple of 4),
-// `ray` the group's ray (-1: none) of positions [beg, end), `S` its depth
-// behind the chunk; lane i's `my_beg` is the first position of ray i.  The
-// product so far stays in rl->T (it takes no register of the blob loop's).
+// One chunk of every group, called by the whole warp: `f` the lane's factors (1
+// for padding), `q` its first position (a multiple of 4), `on` whether the
+// group's ray, `ray` of positions [beg, end), is faint, `S` its depth behind
+// the chunk; lane i's `my_beg` is the first position of ray i.  The product so
+// far stays in rl->T (it takes no register of the blob loop's).
 __device__ __forceinline__ void faint_chunk(float* ring, RayLen* rl, const float2 f[kPairs],
-                                            int ray, int q, int beg, int end, int my_beg,
+                                            bool on, int ray, int q, int beg, int end, int my_beg,
                                             float S) {
   static_assert(kPairs == 2, "one 16-byte store per lane");
-  const bool on = ray >= 0 && S < kFaintDepth;
-  const int task = __shfl_sync(kFieldFull, my_beg, ray & ~(kFaintRays - 1));
   const int gl = threadIdx.x & (kGroupLanes - 1);
   if (on)
     *reinterpret_cast<float4*>(ring + (unsigned)q % kRing) =
         make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+  on = on && !(fabsf(S) < kNoDepth);
+  // where every factor so far is 1 (few blobs, rays that miss them) no product is needed
+  // (unbounded frame without blobs: 458 -> 349 us, with four 519 -> 406)
+  if (!__any_sync(kFieldFull, on)) return;
+  const int task = __shfl_sync(kFieldFull, my_beg, ray & ~(kFaintRays - 1));
   __syncwarp();
   const int base = q - kPerLane * gl;  // the chunk's positions
   const int to = min(base + kChunk, end);

@@ -70,7 +70,7 @@ __device__ __forceinline__ int number_runs(uint2* sr, int nr) {
   return pos;
 }
 
-template <int kMode, bool kStore, bool kMany>
+template <int kMode, bool kStore, int kForm>
 __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R, GridDev g,
     LatticeDev lat, const uint8_t* __restrict__ nruns,
@@ -79,13 +79,13 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
   // field_layout, then [kRenderWarps][R][kRunStride] runs
   extern __shared__ __align__(16) unsigned char smem[];
   const FieldLayout L = field_layout(G, kRenderWarps, R, 0);
-  stage_blobs(smem, L, field, G);
+  stage_blobs<kForm>(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int grp = lane / kGroupLanes, gl = lane & (kGroupLanes - 1);
   const int64_t task = (int64_t)blockIdx.x * kRenderWarps + wib, first = task * R;
   if (first >= n) return;  // uniform per warp; no block barrier follows
-  FieldWarp<kMany> fw;
+  FieldWarp<kForm> fw;
   fw.init(smem, L);
   uint2* sr = reinterpret_cast<uint2*>(smem + L.bytes) + wib * R * kRunStride;
 
@@ -232,11 +232,12 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     BlobSums sums;
     sums_clear(sums);
     sum_blobs(smem, fw.recs + L.list, len, t, sums);
-    if constexpr (kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
+    if constexpr (kForm == kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
       evals += (unsigned)kept * (unsigned) min(kChunk, W - q);
     float2 f[kPairs];
-    if (shade_chunk(sums, dt, ray, acc, f)) acc.T *= faint_product(f);  // uniform
+    const bool faint = shade_chunk(sums, dt, ray, acc, f);
+    faint_product(f, faint, acc);
     q += kChunk;
     const bool round_over = ray >= 0 && q - kPerLane * gl >= W;
     bool done = round_over && k_next >= lat.K;
@@ -291,7 +292,7 @@ int launch_field(const WalkArgs& w, const uint8_t* nr, const uint2* runs, const 
   const size_t smem = field_layout(G, kRenderWarps, R, 0).bytes +
                       (size_t)kRenderWarps * R * kRunStride * sizeof(uint2);
   const auto kern =
-      G <= kAllBlobs ? render_kernel<kMode, kStore, false> : render_kernel<kMode, kStore, true>;
+      G <= kAllBlobs ? render_kernel<kMode, kStore, kSome> : render_kernel<kMode, kStore, kMany>;
   if (smem > 48 * 1024)
     HDDA_CUDA_TRY(
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -89,7 +89,12 @@ struct RayRec {
 // What else a ray keeps: |d|, the rounding margin of distances to its line, and the
 // transmittance of a faint ray (faint_chunk).
 struct RayLen {
-  float len, margin, T, unused;
+  float len, margin;
+  union {
+    float T;
+    int next_w;  // render.cu: the samples of the ray's next round
+  };
+  int next_k;    // and where the one after it resumes
 };
 
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
@@ -247,7 +252,7 @@ __device__ __forceinline__ void make_ray_rec(RayRec* rr, RayLen* len, const floa
   const bool moves = dd > 1e-30f;
   rr->base = make_float4(b[0], b[1], b[2], tb);
   rr->dir = make_float4(d[0], d[1], d[2], moves ? 1.f / dd : 0.f);
-  *len = RayLen{moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm), 1.f, 0.f};
+  *len = RayLen{moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm), {1.f}, 0};
 }
 
 // sqrt(x), approximately, rounded up and its low 8 bits replaced by a blob's

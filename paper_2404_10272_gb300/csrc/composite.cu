@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
     }
     float2 t[kPairs], dt[kPairs];
     float lo, hi;
-    chunk_params(a, b, tb, q - beg, end - beg, t, dt, lo, hi);
+    chunk_params<false>(a, b, tb, q - beg, end - beg, t, dt, lo, hi);
     int kept;
     const int len = fw.cull(L, G, lo, hi, kept);
     q += kChunk;

@@ -667,7 +667,9 @@ __device__ __forceinline__ void faint_chunk(float* ring, RayLen* rl, const float
 // and the group's range of the former.  `rel` is the lane's first position
 // in the ray (negative before its first sample) and `count` the ray's
 // samples: positions outside [0, count) become padding (length 0, a parameter
-// within the range).
+// within the range).  kAscend: the ray's samples ascend and the group's first
+// one is one of them, so its first and last one bound the range.
+template <bool kAscend>
 __device__ __forceinline__ void chunk_params(const float2 a[kPairs], const float2 b[kPairs],
                                              float tb, int rel, int count, float2 t[kPairs],
                                              float2 dt[kPairs], float& lo, float& hi) {
@@ -677,32 +679,38 @@ __device__ __forceinline__ void chunk_params(const float2 a[kPairs], const float
     t[h] = __fadd2_rn(__fadd2_rn(a[h], B), __fadd2_rn(b[h], B));
     dt[h] = make_float2(b[h].x - a[h].x, b[h].y - a[h].y);
   }
+  if constexpr (kAscend) lo = __shfl_sync(kFieldFull, t[0].x, 0, kGroupLanes);
   const bool part = rel < 0 || rel + kPerLane > count;
   const bool any = __any_sync(kFieldFull, part);
   if (any) {  // uniform
+    const float pad = kAscend ? lo : NAN;  // NaN: left out of the range
 #pragma unroll
     for (int h = 0; h < kPairs; ++h) {
       const bool i0 = (unsigned)(rel + 2 * h) < (unsigned)count;
       const bool i1 = (unsigned)(rel + 2 * h + 1) < (unsigned)count;
-      t[h] = make_float2(i0 ? t[h].x : NAN, i1 ? t[h].y : NAN);  // NaN: left out of the range
+      t[h] = make_float2(i0 ? t[h].x : pad, i1 ? t[h].y : pad);
       dt[h] = make_float2(i0 ? dt[h].x : 0.f, i1 ? dt[h].y : 0.f);
     }
   }
-  lo = fminf(t[0].x, t[0].y);
   hi = fmaxf(t[0].x, t[0].y);
 #pragma unroll
-  for (int h = 1; h < kPairs; ++h) {
-    lo = fminf(lo, fminf(t[h].x, t[h].y));
-    hi = fmaxf(hi, fmaxf(t[h].x, t[h].y));
-  }
+  for (int h = 1; h < kPairs; ++h) hi = fmaxf(hi, fmaxf(t[h].x, t[h].y));
+  if constexpr (kAscend) {
+    const int last = count - 1 - rel + kPerLane * (threadIdx.x & (kGroupLanes - 1));
+    hi = __shfl_sync(kFieldFull, hi, min(last, kChunk - 1) / kPerLane, kGroupLanes);
+  } else {
+    lo = fminf(t[0].x, t[0].y);
 #pragma unroll
-  for (int o = 1; o < kGroupLanes; o <<= 1) {
-    lo = fminf(lo, __shfl_xor_sync(kFieldFull, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(kFieldFull, hi, o));
-  }
-  if (any) {
+    for (int h = 1; h < kPairs; ++h) lo = fminf(lo, fminf(t[h].x, t[h].y));
 #pragma unroll
-    for (int h = 0; h < kPairs; ++h) t[h] = make_float2(fmaxf(t[h].x, lo), fmaxf(t[h].y, lo));
+    for (int o = 1; o < kGroupLanes; o <<= 1) {
+      lo = fminf(lo, __shfl_xor_sync(kFieldFull, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(kFieldFull, hi, o));
+    }
+    if (any) {
+#pragma unroll
+      for (int h = 0; h < kPairs; ++h) t[h] = make_float2(fmaxf(t[h].x, lo), fmaxf(t[h].y, lo));
+    }
   }
 }
 

@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
     }
     float2 t[kPairs], dt[kPairs];
     float lo, hi;
-    chunk_params(a, b, tb, q, W, t, dt, lo, hi);
+    chunk_params<true>(a, b, tb, q, W, t, dt, lo, hi);
     int kept;
     const int len = fw.cull(L, G, lo, hi, kept);
     BlobSums sums;

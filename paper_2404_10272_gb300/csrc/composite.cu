@@ -15,6 +15,10 @@ namespace hdda {
 namespace {
 
 constexpr int kWarpsPerCta = 4;
+// Records per group in 64ths of a field of many blobs.  Not 32: with that the form for up to 64
+// blobs, which does not use it, is compiled with 28 bytes of spills instead of 4 and is 3 % slower
+// (object frame 307 and 317 us); here 32 and 33 are equally fast.
+constexpr int kRoom64 = 33;
 
 // Blob evaluations (sample x kept blob), counted only while profiling.
 __device__ unsigned long long g_blob_evals;
@@ -55,13 +59,13 @@ __device__ __forceinline__ void load_lane(const float* __restrict__ t0, const fl
 }
 
 template <bool kVec, int kForm>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, 6) composite_kernel(
+__global__ void __launch_bounds__(kWarpsPerCta * 32, kForm == kMany ? 5 : 6) composite_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R,
     const int64_t* __restrict__ offsets, const float* __restrict__ t0,
     const float* __restrict__ t1, const float* __restrict__ field, int G,
     float* __restrict__ rgba, bool count_evals) {
   extern __shared__ __align__(16) unsigned char smem[];  // field_layout
-  const FieldLayout L = field_layout(G, kWarpsPerCta, R, kForm == kMany ? 0 : kRing);
+  const FieldLayout L = field_layout<kRoom64>(G, kWarpsPerCta, R, kForm == kMany ? 0 : kRing);
   stage_blobs<kForm>(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -199,7 +203,7 @@ extern "C" int hdda_composite(const float* rays_o, const float* rays_d, int64_t 
   const int64_t blocks = (warps + kWarpsPerCta - 1) / kWarpsPerCta;
   if (blocks > INT32_MAX) return set_error(HDDA_ERR_INVALID_ARG, "too many rays");
   const unsigned grid = (unsigned)blocks;
-  const FieldLayout L = field_layout(n_gauss, kWarpsPerCta, R, n_gauss <= kAllBlobs ? kRing : 0);
+  const FieldLayout L = field_layout<kRoom64>(n_gauss, kWarpsPerCta, R, n_gauss <= kAllBlobs ? kRing : 0);
   const bool vec = ((reinterpret_cast<uintptr_t>(t0) | reinterpret_cast<uintptr_t>(t1)) & 15) == 0;
   const auto kern = n_gauss <= kFewBlobs
                         ? (vec ? composite_kernel<true, kFew> : composite_kernel<false, kFew>)

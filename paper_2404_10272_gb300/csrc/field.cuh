@@ -106,11 +106,15 @@ struct RayLen {
 // record, offset of its colour}, and `ring` factors of a faint ray.
 //
 // Up to kAllBlobs blobs every one has a record in every group.  A larger field
-// would leave too few warps on an SM that way (eight at 256 blobs); there a
-// group has room for 5/8 of them, and a ray within reach of more takes each
-// chunk in passes (FieldWarp::more, kMany).  An 800 x 800 object frame takes
-// 0.62 -> 0.48 ms at 128 blobs and 1.62 -> 1.29 ms at 256 by this (0.45 and 1.22
-// since).
+// would leave too few warps on an SM that way; there a group has room for about
+// half of them (99 % of the rays of an object or an unbounded frame are within
+// reach of less), and a ray within reach of more takes each chunk in passes
+// (FieldWarp::more, kMany).  Shared memory then lets at most five CTAs on an SM
+// from 160 blobs on, so the kernels have the registers of five (96): at 80 they
+// spilled 110 to 160 bytes.  With room for 5/8 and 80 registers, and so (us): 128
+// blobs, object frame 550 and 477, unbounded 1125 and 943; 200 blobs 996 and 741,
+// 2088 and 1486; 256 blobs 1235 and 1016, 2608 and 2085.  (Distances in space,
+// without records, took 661 and 1161, 1002 and 1689, 1356 and 2403.)
 constexpr int kAllBlobs = 64;
 
 // Up to kFewBlobs blobs the compositor's groups each set up their own ray (kFew).
@@ -124,9 +128,10 @@ struct FieldLayout {
 };
 
 // `ring`: factors of faint rays kept per group.
+template <int kRoom64>
 __host__ __device__ inline FieldLayout field_layout(int G, int warps, int R, int ring) {
   FieldLayout L;
-  L.cap = G <= kAllBlobs ? G : (5 * G / 8 > kAllBlobs ? 5 * G / 8 : kAllBlobs);
+  L.cap = G <= kAllBlobs ? G : (kRoom64 * G / 64 > kAllBlobs ? kRoom64 * G / 64 : kAllBlobs);
   L.col = (uint32_t)field_pairs(G) * kPairBytes;
   L.warp0 = L.col + ((uint32_t)G + 2u) * sizeof(float4);
   L.len = (uint32_t)R * sizeof(RayRec);

@@ -37,6 +37,7 @@ namespace hdda {
 namespace {
 
 constexpr int kRenderWarps = 4;
+constexpr int kRoom64 = 32;  // records per group in 64ths of a field of many blobs
 constexpr uint32_t kNoRun = 0x7fffffffu;
 constexpr unsigned kWalked = 1u, kOther = 2u;
 constexpr int kRunStride = kMaxRuns + 1;  // per ray: odd, so the groups' searches hit other banks
@@ -75,7 +76,7 @@ __device__ __forceinline__ int number_runs(uint2* sr, int nr) {
 }
 
 template <int kMode, bool kStore, int kForm>
-__global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
+__global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) render_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R, GridDev g,
     LatticeDev lat, const uint8_t* __restrict__ nruns,
     const uint2* __restrict__ runs, const float* __restrict__ field, int G,
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 6) render_kernel(
   // field_layout, then per warp [R + kGroups][kRunStride] runs: the rays' and, per group, those
   // of its ray's next round
   extern __shared__ __align__(16) unsigned char smem[];
-  const FieldLayout L = field_layout(G, kRenderWarps, R, 0);
+  const FieldLayout L = field_layout<kRoom64>(G, kRenderWarps, R, 0);
   stage_blobs<kForm>(smem, L, field, G);
   __syncthreads();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -302,7 +303,7 @@ int launch_field(const WalkArgs& w, const uint8_t* nr, const uint2* runs, const 
   const int R = field_task_rays(w.n);
   const int64_t warps = (w.n + R - 1) / R;
   const unsigned nb = (unsigned)((warps + kRenderWarps - 1) / kRenderWarps);
-  const size_t smem = field_layout(G, kRenderWarps, R, 0).bytes +
+  const size_t smem = field_layout<kRoom64>(G, kRenderWarps, R, 0).bytes +
                       (size_t)kRenderWarps * (R + kGroups) * kRunStride * sizeof(uint2);
   const auto kern =
       G <= kAllBlobs ? render_kernel<kMode, kStore, kSome> : render_kernel<kMode, kStore, kMany>;

@@ -518,8 +518,11 @@ int hdda_traverse_composite(const float* rays_o, const float* rays_d, int64_t n_
  *                          by two CUDA events recorded on its stream (one
  *                          event pair per launch)
  *   HDDA_PROFILE_COUNTERS  the compositors count blob evaluations (sample x
- *                          kept blob), one atomic add per ray; this is
- *                          extra device work, so time with the timers alone
+ *                          kept blob), with an atomic add per ray of
+ *                          hdda_composite (whose count of a single ray wraps
+ *                          at 2^32) and one per 32 samples of a ray of the
+ *                          others; this is extra device work, so time with
+ *                          the timers alone
  * hdda_profiler_enable(flags) sets both switches (0 turns everything off).
  * hdda_profiler_read synchronises on the recorded events, writes up to `cap`
  * per-kernel aggregates (HOST array) and clears them; *n_out (HOST)

@@ -157,7 +157,6 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
   unsigned ahead = 0;  // kWalked: the next round is there; kOther: this one is in the group's runs
   float tb = 0.f;
   int64_t gofs = 0;
-  unsigned evals = 0;  // of the ray in work
   RayAcc acc;
   acc_clear(acc);
   rgba += 4 * first;
@@ -241,7 +240,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
     sum_blobs(smem, fw.recs + L.list, len, t, sums);
     if constexpr (kForm == kMany) fw.more(L, G, ray, lo, hi, t, sums, kept);
     if (count_evals && ray >= 0 && gl == 0)
-      evals += (unsigned)kept * (unsigned) min(kChunk, W - q);
+      atomicAdd(&g_render_evals, (unsigned long long)(kept * min(kChunk, W - q)));
     float2 f[kPairs];
     const bool faint = shade_chunk(sums, dt, ray, acc, f);
     faint_product(f, faint, acc);
@@ -284,8 +283,6 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
         ahead = 0;
         fw.release();
         acc_clear(acc);
-        if (count_evals && gl == 0) atomicAdd(&g_render_evals, (unsigned long long)evals);
-        evals = 0;
       }
     }
     __syncwarp();  // the group's lists, records and runs may be overwritten

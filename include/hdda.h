@@ -443,9 +443,12 @@ void hdda_batch_free(hdda_batch* batch);
  *     c     = sum_g a_g exp(...) rgb_g / sigma      (0 when sigma == 0)
  *     alpha = 1 - exp(-sigma (t1 - t0)) ;  C += T alpha c ;  T *= 1 - alpha
  * and rgba_out[r] = (C, 1 - T): black background, no early termination.
- *   rays_o, rays_d  device float [n_rays][3]
+ *   rays_o, rays_d  device float [n_rays][3]; directions of any length from
+ *                   1e-36 to 1e36 (t is in units of it), or zero
  *   offsets         device int64 [n_rays + 1] (as written by a traversal)
- *   t0, t1          device float samples
+ *   t0, t1          device float samples; 16-byte aligned, they are read in
+ *                   whole 16-byte lines, also the line of sample offsets[0]
+ *                   where that is not its first
  *   field           device float [n_gauss][8] = mu_x, mu_y, mu_z, s, a, r, g, b,
  *                   with s > 0 and a >= 0.  A blob is skipped for a group of
  *                   up to 32 samples of one ray when it lies farther than 7 s from

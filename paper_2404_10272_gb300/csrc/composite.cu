@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kWarpsPerCta * 32, kForm == kMany ? 5 : 6) com
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, base_param(smem, L, G, o, d, ta, te));
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, smem, L, G, o, d, ta, te);
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
   }

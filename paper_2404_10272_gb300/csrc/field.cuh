@@ -47,7 +47,7 @@
 // when several are idle (0 to 5 % slower).
 //
 // Rounding.  Ray parameters are taken relative to a base parameter near the
-// blobs (base_param), where the base point is rounded once, so t* and p carry
+// blobs (make_ray_rec), where the base point is rounded once, so t* and p carry
 // the rounding of coordinates near the blobs, not of the origin's.  Every
 // product-sum is an explicit fused multiply-add, so the arithmetic does not
 // depend on the translation unit's contraction flags.
@@ -79,22 +79,21 @@ constexpr float kLog2e = 1.4426950408889634f;
 __host__ __device__ inline int field_pairs(int G) { return (G + 63) / 64 * 32; }
 constexpr uint32_t kPairBytes = 3 * sizeof(float4) + sizeof(float2);
 
-// A ray as setup_ray reads it: base point and base parameter, direction and
-// 1 / |d|^2; beside it a RayLen.
+// A ray as setup_ray reads it: base point and base parameter, direction e = s d
+// and 1 / |e|^2 (dir_scale); beside it a RayLen.
 struct RayRec {
   float4 base;  // o + tb d, tb
-  float4 dir;   // d, 1 / |d|^2
+  float4 dir;   // e, 1 / |e|^2
 };
 
-// What else a ray keeps: |d|, the rounding margin of distances to its line, and the
-// transmittance of a faint ray (faint_chunk).
-struct RayLen {
-  float len, margin;
+// What else a ray keeps.
+struct __align__(16) RayLen {
+  float len, margin;  // |e|; the rounding margin of distances to its line
+  float half;         // 1 / (2 s): from half a parameter along e to one along d
   union {
-    float T;
-    int next_w;  // render.cu: the samples of the ray's next round
+    float T;          // a faint ray's transmittance (faint_chunk)
+    int next_w;       // render.cu: the samples of the ray's next round
   };
-  int next_k;    // and where the one after it resumes
 };
 
 // Dynamic shared memory of a compositing CTA of `warps` warps over G blobs,
@@ -187,21 +186,6 @@ __device__ __forceinline__ void stage_blobs(unsigned char* smem, const FieldLayo
   }
 }
 
-// The base parameter of a ray whose samples lie between ta and tb: where it
-// passes nearest to the blobs' mean centre.  Parameters and distances are exact
-// to the rounding of numbers of the size of their difference from the base,
-// and most of a field's weight lies near its middle, while a ray's samples may
-// reach far beyond it (a four-level cascade: with the middle of the samples as
-// the base the error against binary64 was up to 1.7 times as large).
-__device__ __forceinline__ float base_param(const unsigned char* smem, const FieldLayout& L, int G,
-                                            const float o[3], const float d[3], float ta,
-                                            float tb) {
-  const float4 m = reinterpret_cast<const float4*>(smem + L.col)[G + 1];
-  const float w = fmaf(m.x - o[0], d[0], fmaf(m.y - o[1], d[1], (m.z - o[2]) * d[2]));
-  const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
-  return fminf(fmaxf(__fdividef(w, dd), fminf(ta, tb)), fmaxf(ta, tb));
-}
-
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -240,11 +224,34 @@ __device__ __forceinline__ void acc_clear(RayAcc& a) {
   a.r = a.g = a.b = splat(0.f);
 }
 
-// Fills the RayRec of one ray (one lane per ray): tb is any parameter
-// (base_param).
-__device__ __forceinline__ void make_ray_rec(RayRec* rr, RayLen* len, const float o[3],
-                                             const float d[3], float tb) {
-  if (!(fabsf(tb) < 1e30f)) tb = 0.f;
+// A power of two that brings a direction of extreme length to one whose square
+// is a normal number; 1 for lengths from 1e-15 to 1e15.
+__device__ __forceinline__ float dir_scale(const float d[3]) {
+  const float m = fmaxf(fabsf(d[0]), fmaxf(fabsf(d[1]), fabsf(d[2])));
+  if (!(m > 0.f) || (m > 1e-15f && m < 1e15f)) return 1.f;
+  const int x = min(max((int)(__float_as_uint(m) >> 23) - 127, -126), 126);
+  return __uint_as_float((uint32_t)(127 - x) << 23);
+}
+
+// Fills the RayRec and RayLen of one ray (one lane per ray) whose samples lie
+// between ta and te.
+//
+// The base parameter is where the ray passes nearest to the blobs' mean centre.
+// Parameters and distances are exact to the rounding of numbers of the size of
+// their difference from the base, and most of a field's weight lies near its
+// middle, while a ray's samples may reach far beyond it (a four-level cascade:
+// with the middle of the samples as the base the error against binary64 was up
+// to 1.7 times as large).
+__device__ __forceinline__ void make_ray_rec(RayRec* rr, RayLen* rl, const unsigned char* smem,
+                                             const FieldLayout& L, int G, const float o[3],
+                                             const float d[3], float ta, float te) {
+  const float4 m = reinterpret_cast<const float4*>(smem + L.col)[G + 1];
+  const float s = dir_scale(d);
+  const float e[3] = {d[0] * s, d[1] * s, d[2] * s};
+  const float w = fmaf(m.x - o[0], e[0], fmaf(m.y - o[1], e[1], (m.z - o[2]) * e[2]));
+  const float ee = fmaf(e[0], e[0], fmaf(e[1], e[1], e[2] * e[2]));
+  float tb = fminf(fmaxf(__fdividef(w, ee) * s, fminf(ta, te)), fmaxf(ta, te));
+  if (!(fabsf(tb) < INFINITY)) tb = 0.f;
   float b[3];
   float om = 0.f, bm = 0.f;
 #pragma unroll
@@ -253,11 +260,13 @@ __device__ __forceinline__ void make_ray_rec(RayRec* rr, RayLen* len, const floa
     om = fmaxf(om, fabsf(o[c]));
     bm = fmaxf(bm, fabsf(b[c]));
   }
-  const float dd = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
-  const bool moves = dd > 1e-30f;
+  const bool moves = ee > 0.f;
   rr->base = make_float4(b[0], b[1], b[2], tb);
-  rr->dir = make_float4(d[0], d[1], d[2], moves ? 1.f / dd : 0.f);
-  *len = RayLen{moves ? sqrtf(dd) : 0.f, 2e-5f * (om + bm), {1.f}, 0};
+  rr->dir = make_float4(e[0], e[1], e[2], moves ? 1.f / ee : 0.f);
+  rl->len = moves ? sqrtf(ee) : 0.f;
+  rl->margin = 2e-5f * (om + bm);
+  rl->half = 0.5f / s;
+  rl->T = 1.f;
 }
 
 // sqrt(x), approximately, rounded up and its low 8 bits replaced by a blob's
@@ -290,7 +299,7 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
   const int lane = threadIdx.x & (w - 1), first = (threadIdx.x & 31) - lane, np = field_pairs(G);
   const unsigned mine = (kFieldFull >> (32 - w)) << first;
   const float4 B = rr->base, D = rr->dir;
-  const float2 len = *reinterpret_cast<const float2*>(rl);  // |d|, margin
+  const float4 len = *reinterpret_cast<const float4*>(rl);  // |e|, margin, 1 / (2 s)
   const float2 dx = splat(D.x), dy = splat(D.y), dz = splat(D.z), nw = splat(-D.w);
   int n = 0;
   for (; q0 < G; q0 += 2 * w) {
@@ -312,7 +321,7 @@ __device__ __forceinline__ int setup_ray(const unsigned char* smem, int G, const
     const float2 hl = __ffma2_rn(rc, splat(len.y), reach);
     const float2 lim2 = __ffma2_rn(hl, hl, make_float2(-cp2.x, -cp2.y));
     const float2 k = __fmul2_rn(rc, splat(len.x));
-    const float2 hk = __fmul2_rn(splat(0.5f), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
+    const float2 hk = __fmul2_rn(splat(len.z), k), b = __fmul2_rn(make_float2(-k.x, -k.y), ts);
     const float2 e = __fadd2_rn(cp2, make_float2(-AK.x, -AK.y));
     const int q = q0 + lane;
     const bool near0 = on && lim2.x >= 0.f && q < G, near1 = on && lim2.y >= 0.f && q + w < G;

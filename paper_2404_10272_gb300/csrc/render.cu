@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
       o[c] = __ldg(ro + 3 * r + c);
       d[c] = __ldg(rd + 3 * r + c);
     }
-    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, o, d, base_param(smem, L, G, o, d, ta, te));
+    make_ray_rec(fw.rays(L) + lane, fw.lens(L) + lane, smem, L, G, o, d, ta, te);
     my_w = number_runs(sr + lane * kRunStride, nr);
   } else if (has_ray) {
     reinterpret_cast<float4*>(rgba)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
     bool done = round_over && k_next >= lat.K;
     const bool more = round_over && !done;  // another round of runs
     if (__any_sync(kFull, more)) {
-      RayLen* const rl = fw.lens(L) + max(ray, 0);  // its T and the last word are free here
+      RayLen* const rl = fw.lens(L) + max(ray, 0);  // its T is free here
       if (__any_sync(kFull, more && !(ahead & kWalked))) {
         // One lane per ray walks on, for every group with runs left and not only for the one
         // that needs them now: a walk is a chain that keeps the warp waiting.
@@ -261,16 +261,17 @@ __global__ void __launch_bounds__(kRenderWarps * 32, kForm == kMany ? 5 : 6) ren
           load_ray(ro, rd, first + ray, ry);
           const LatHdr h = lat_hdr(lat);
           int nr2 = 0;
-          rl->next_k = walk_from<kMode, false>(g, global_tabs(g, lat), lat, h, ry, k_next, mr, 1, nr2);
+          const int kn = walk_from<kMode, false>(g, global_tabs(g, lat), lat, h, ry, k_next, mr, 1, nr2);
           rl->next_w = number_runs(mr, nr2);
+          mr[kMaxRuns].x = (uint32_t)kn;  // where it resumes: that slot holds no run
         }
         __syncwarp();
       }
       if (more) {
         gofs += W;
         W = rl->next_w;
-        k_next = rl->next_k;
         ahead ^= kWalked | kOther;
+        k_next = (int)sr[(ahead & kOther ? R + grp : ray) * kRunStride + kMaxRuns].x;
         q = kPerLane * gl;
         done = W == 0;
       }

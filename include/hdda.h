@@ -19,6 +19,11 @@
  *     are stream-ordered and return before the GPU work finishes, except
  *     where a host value is returned (noted per call): those synchronise the
  *     stream once.
+ *   - Scratch comes from a stream-ordered memory pool of the library's own, one
+ *     per device ("the stream-ordered allocator" below).  Between calls the
+ *     pool keeps up to 1 GiB of it, which other allocators on the device
+ *     cannot use, as long as the device has a grid or a batch; with the last
+ *     of them all of it goes back, at the latest at the next synchronisation.
  *   - Every call returns an hdda_status; 0 is success.  On failure
  *     hdda_last_error() gives a message (thread-local).  No C++ exception
  *     crosses this boundary.  A failed call leaves outputs unspecified.

@@ -39,8 +39,9 @@ void clear_error() { g_last_error[0] = '\0'; }
 // mapped its scratch anew: 300 us for a 9,216-ray frame whose kernels take 75,
 // and 0.65 against 0.25 ms for an 800 x 800 sampler call waited for.  The bound holds a
 // call of seven million rays, or several smaller ones in flight at once; more
-// is given back at the next synchronisation, and all of it with the device's
-// last grid and batch.
+// is given back at the next synchronisation.  While the device has no grid and
+// no batch the bound is zero: what the last of them still had in flight goes
+// back at the next synchronisation too.
 namespace {
 constexpr int kMaxPoolDevices = 64;
 constexpr uint64_t kPoolKeep = 1ull << 30;
@@ -61,12 +62,6 @@ cudaError_t pool_of(int dev, cudaMemPool_t* out) {
     cudaMemPool_t pool = nullptr;
     cudaError_t e = cudaMemPoolCreate(&pool, &props);
     if (e != cudaSuccess) return e;
-    uint64_t keep = kPoolKeep;
-    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e != cudaSuccess) {
-      cudaMemPoolDestroy(pool);
-      return e;
-    }
     g_pools[dev] = pool;
   }
   *out = g_pools[dev];
@@ -99,8 +94,15 @@ void scratch_users(int device, int change) {
   // made here, where memory is allocated anyway, and not first inside a stream capture
   if (change > 0 && pool_of(device, &pool) != cudaSuccess) cudaGetLastError();
   std::lock_guard<std::mutex> lock(g_pool_mu);
+  const bool had = g_pool_users[device] > 0;
   g_pool_users[device] += change;
-  if (g_pool_users[device] == 0 && g_pools[device]) cudaMemPoolTrimTo(g_pools[device], 0);
+  const bool has = g_pool_users[device] > 0;
+  pool = g_pools[device];
+  if (had == has || !pool) return;
+  uint64_t keep = has ? kPoolKeep : 0;
+  cudaError_t e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  if (e == cudaSuccess && !has) e = cudaMemPoolTrimTo(pool, 0);
+  if (e != cudaSuccess) cudaGetLastError();  // only how much is kept depends on it
 }
 
 int sm_count(int device) {

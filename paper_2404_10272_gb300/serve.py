@@ -35,6 +35,9 @@ Per request, in the slot's stream:
      walk and the run-level compositor render it;
   3. the frame is copied back to pinned host memory.
 
+The budget counts what admitted requests hold; beside it the library keeps up to
+1 GiB of scratch between calls (include/hdda.h).
+
 Latency runs from arrival to the frame in host memory.  The library calls
 release the GIL, so the slots' GPU work overlaps.
 

@@ -118,8 +118,11 @@ typedef struct {
     int32_t reserved;
     int64_t n_leaves;    /* VDB: stored 8^3 leaf bitmasks (partial blocks)  */
     int64_t n_tiles;     /* VDB: fully occupied blocks stored as tile bits  */
-    int64_t bytes;       /* bytes the traversal reads: level table,
-                            index thresholds, masks and leaves (Table 3)    */
+    int64_t bytes;       /* the structure of Table 3: level table, index
+                            thresholds (HDDA_ARRAY_THRESHOLDS), masks and
+                            leaves.  The traversal reads the thresholds in
+                            a form for both directions instead, 2 res + 128
+                            floats per axis and level, which is not counted */
     int64_t dense_bytes; /* levels * ceil(res^3 / 32) * 4: the dense bit
                             array the paper starts from (Table 3 caption)   */
     int64_t map_bytes;   /* VDB: the region map HDDA reads with refinement

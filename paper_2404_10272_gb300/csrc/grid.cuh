@@ -56,7 +56,7 @@ struct hdda_grid {
         g.lv[l].s[c] = scale[l][c];
       }
     }
-    g.thr = thr; g.mthr = mthr; g.bits = bits; g.child = child; g.tile = tile;
+    g.mthr = mthr; g.bits = bits; g.child = child; g.tile = tile;
     g.prefix = prefix; g.nstate = nstate; g.leaves = leaves;
     g.nsuper = nsuper; g.lsub = lsub; g.rmap = rmap;
     g.check = hdda::region_checks_on() ? 1 : 0;

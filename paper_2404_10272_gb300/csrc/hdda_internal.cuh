@@ -68,8 +68,7 @@ struct GridDev {
   int L, R, B, N;
   int W;                     // dense bit words per level
   LevelDev lv[kMaxLevels];
-  const float* thr;          // [L][3][R+1] exact index thresholds
-  const float* mthr;         // [L][3][mthr_stride(R)] the same as mirrored upper bounds
+  const float* mthr;         // [L][3][mthr_stride(R)] exact index thresholds as mirrored upper bounds
   const uint32_t* bits;      // dense: [L][W]
   const uint32_t* child;     // vdb: [L*N^3][128]
   const uint32_t* tile;      // vdb: [L*N^3][128]

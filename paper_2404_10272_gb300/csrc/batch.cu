@@ -78,9 +78,13 @@ __device__ __forceinline__ void warp_copy(T* dst, const T* src) {
 
 // Bounded by instruction issue (73 % of cycles issue, 22 of 32 lanes active).
 // What a job's rays share is read from shared memory as needed and the
-// registers are held to 64, so 32 warps fit an SM instead of 24: 64 cameras of
-// up to 800 x 800 pixels (12 M rays, 600 M samples) took 3960 us in all with 75
-// registers, 3877 with 64.
+// registers are held to 64, so 32 warps fit an SM instead of 24, at the price of
+// spills (16 bytes; 80 to 176 with the plain tree).  64 cameras of up to 800 x 800
+// pixels (12 M rays, 600 M samples) take 3832 us in all with 64 registers and
+// 3903 without the bound, over the plain tree 6094 and 6205, over dense grids
+// 9421 and 9371, in blocks of 512 threads 3824 and 4842.  Batches that do not
+// fill the chip have no use for the warps: one 800 x 800 camera takes 238 and
+// 218 us, eight of 64 x 64 pixels 112 and 105.
 template <int kMode, int kBlock, bool kSkip, bool kCheck>
 __global__ void __launch_bounds__(kBlock, 1024 / kBlock) batch_walk_kernel(
     const JobDev* __restrict__ jobs, const int64_t* __restrict__ tile0, int J, int64_t T,

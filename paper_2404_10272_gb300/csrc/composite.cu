@@ -14,7 +14,8 @@
 namespace hdda {
 namespace {
 
-constexpr int kWarpsPerCta = 4;
+constexpr int kWarpsPerCta = 4;  // CTAs per SM: 6 by registers (80); up to 32 blobs 7 (72: object
+                                 // frame over 16 blobs 228 -> 220 us); over 64, see kAllBlobs
 // Records per group in 64ths of a field of many blobs.  Not 32: with that the form for up to 64
 // blobs, which does not use it, is compiled with 28 bytes of spills instead of 4 and is 3 % slower
 // (object frame 307 and 317 us); here 32 and 33 are equally fast.
@@ -59,7 +60,7 @@ __device__ __forceinline__ void load_lane(const float* __restrict__ t0, const fl
 }
 
 template <bool kVec, int kForm>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, kForm == kMany ? 5 : 6) composite_kernel(
+__global__ void __launch_bounds__(kWarpsPerCta * 32, kForm == kMany ? 5 : kForm == kFew ? 7 : 6) composite_kernel(
     const float* __restrict__ ro, const float* __restrict__ rd, int64_t n, int R,
     const int64_t* __restrict__ offsets, const float* __restrict__ t0,
     const float* __restrict__ t1, const float* __restrict__ field, int G,
@@ -198,7 +199,10 @@ extern "C" int hdda_composite(const float* rays_o, const float* rays_d, int64_t 
     return set_error(HDDA_ERR_INVALID_ARG, "NULL pointer");
   if (reinterpret_cast<uintptr_t>(rgba_out) % 16 != 0)
     return set_error(HDDA_ERR_INVALID_ARG, "rgba_out must be 16-byte aligned");
-  const int R = field_task_rays(n_rays);
+  // over up to 16 blobs a task is over soon: of twice as many rays its start weighs less (640,000
+  // rays of 20 samples over 16 blobs 253 -> 222 us, over 32 298 -> 267, but an object frame over 32
+  // 248 -> 262)
+  const int R = field_task_rays(n_rays) * (n_gauss <= 16 && n_rays >= 65536 ? 2 : 1);
   const int64_t warps = (n_rays + R - 1) / R;
   const int64_t blocks = (warps + kWarpsPerCta - 1) / kWarpsPerCta;
   if (blocks > INT32_MAX) return set_error(HDDA_ERR_INVALID_ARG, "too many rays");

@@ -47,3 +47,31 @@ def test_few_blobs(H, G, lengths):
                              torch.from_numpy(field).cuda())).astype(np.float64)
     ref = oracle.composite(o, d, off, t0, t1, field)
     assert np.abs(rgba - ref).max() <= TOL, np.abs(rgba - ref).max()
+
+
+@pytest.mark.parametrize("G", [0, 5, 16, 17])
+def test_large_calls(H, G):
+    # from 65,536 rays on: tasks of 16 rays over up to 16 blobs, of 8 over more; the last one is cut
+    rng = np.random.default_rng(G)
+    n = 65541
+    counts = rng.choice([0, 1, 2, 3, 40], n)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int64)
+    S = int(off[-1])
+    o = rng.uniform(-1.0, 1.0, (n, 3)).astype(np.float32)
+    o[:, 2] -= 2.0
+    d = np.tile(np.array([[0.0, 0.6, 0.8]], np.float32), (n, 1))
+    first = rng.uniform(0.5, 3.0, n).astype(np.float32)
+    k = np.arange(S) - np.repeat(off[:-1], counts)
+    t0 = (np.repeat(first, counts) + 0.02 * k).astype(np.float32)
+    t1 = (t0 + np.float32(0.02)).astype(np.float32)
+    field = np.zeros((G, 8), np.float32)
+    field[:, :3] = rng.uniform(-1.5, 1.5, (G, 3))
+    field[:, 3] = rng.uniform(0.1, 0.3, G)
+    field[:, 4] = rng.uniform(0.5, 50.0, G)
+    field[:, 5:] = rng.uniform(0.0, 1.0, (G, 3))
+    s = H.Samples(torch.from_numpy(off).cuda(), torch.zeros(S, dtype=torch.int32, device="cuda"),
+                  torch.from_numpy(t0).cuda(), torch.from_numpy(t1).cuda(), S)
+    rgba = to_np(H.composite(torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), s,
+                             torch.from_numpy(field).cuda())).astype(np.float64)
+    ref = oracle.composite(o, d, off, t0, t1, field)
+    assert np.abs(rgba - ref).max() <= TOL, np.abs(rgba - ref).max()

@@ -55,18 +55,18 @@ KERNELS_PER_TIMER = {"build_vdb": 4}   # the builder's timer spans four kernels
 PROFILED_COUNTERS = {
     "object": {"hdda_walk": {"l2_hit_pct": 53.7, "active_lanes_of_32": 27.79},
                "hdda_emit": {"l2_hit_pct": 10.7, "active_lanes_of_32": 27.18},
-               "composite": {"l2_hit_pct": 46.9, "active_lanes_of_32": 29.53}},
+               "composite": {"l2_hit_pct": 35.4, "active_lanes_of_32": 29.41}},
     "unbounded": {"hdda_walk": {"l2_hit_pct": 57.5, "active_lanes_of_32": 26.28},
                   "hdda_emit": {"l2_hit_pct": 10.0, "active_lanes_of_32": 30.15},
-                  "composite": {"l2_hit_pct": 38.6, "active_lanes_of_32": 29.96}},
+                  "composite": {"l2_hit_pct": 30.9, "active_lanes_of_32": 29.86}},
 }
 # DRAM bytes (read + write) per launch from ncu of a workload's step on camera 0 (the
 # capture commands are kept with the profile summaries), for the roofline's "traffic"; an
 # entry must be dropped whenever its kernel changes, and a workload without a capture
 # reports none.
 PROFILED_TRAFFIC = {
-    "object": {"hdda_emit": 269_658_880, "hdda_walk": 16_226_048, "composite": 226_914_304},
-    "unbounded": {"hdda_emit": 2_182_256_640, "hdda_walk": 33_935_616, "composite": 1_502_339_072},
+    "object": {"hdda_emit": 269_583_360, "hdda_walk": 16_226_048, "composite": 226_961_664},
+    "unbounded": {"hdda_emit": 2_182_493_696, "hdda_walk": 33_778_688, "composite": 1_502_347_264},
 }
 
 

@@ -33,18 +33,19 @@
 // e^-24.5, about 2e-11 of its amplitude.  Amplitudes must be non-negative
 // (their logarithm is taken).
 //
-// What bounds it: instruction issue and latency (64 % of cycles issue at 24
-// warps per SM; the longest waits are those on the last result and on shared
-// memory).  36 % of the instructions are the blob loop, the rest is per chunk
-// (listing, range, opacities, scan) and per ray (records).  Against two samples per lane of
-// whichever rays come next, with distances in space and colours scanned per
-// chunk, the compositor went from 434 to 297 us on an 800 x 800 object frame
-// and from 2367 to 1460 us on a 1245 x 825 unbounded one.  Tried: four lanes per ray
-// with eight samples each (a quarter fewer instructions, but 14 warps per SM:
+// What bounds it: instruction issue and latency (67 % of cycles issue at 24
+// warps per SM).  36 % of the instructions are the blob loop, the rest is per
+// chunk (listing, range, opacities, scan) and per ray (records).  Against two
+// samples per lane of whichever rays come next, with distances in space and
+// colours scanned per chunk, the compositor went from 432 to 308 us on an 800 x
+// 800 object frame of 64 blobs and from 864 to 658 on a 1245 x 825 unbounded one.
+// Tried, at 64 blobs when they took 297 and 1460 (another camera): four lanes per
+// ray with eight samples each (a quarter fewer instructions, but 14 warps per SM:
 // 20 % slower), 16 lanes' worth of registers saved by loading behind the blob
-// loop (12 % slower), 7 CTAs per SM (spills, 15 % slower), CTAs of 8 to 16
-// tasks that their warps take in turn (5 to 10 % slower), groups refilled only
-// when several are idle (0 to 5 % slower).
+// loop (12 % slower), 7 CTAs per SM (spills, 15 % slower), CTAs of 8 to 16 tasks
+// that their warps take in turn (5 to 10 % slower), groups refilled only when
+// several are idle (0 to 5 % slower).  The layout's offsets as a kernel parameter
+// instead of sums of its sizes: fewer spills, 3 % slower.
 //
 // Rounding.  Ray parameters are taken relative to a base parameter near the
 // blobs (make_ray_rec), where the base point is rounded once, so t* and p carry

@@ -60,7 +60,8 @@
 // from a decoupled look-back.  The allocation-free entry point runs one
 // kernel, onepass_kernel, whose CTAs keep the runs in shared memory and look
 // back right after walking, so its scratch stays a few hundred kilobytes.  A
-// ray with more runs than are kept walks again and writes its own samples.
+// ray with more runs than are kept writes the rest itself: it walks on behind
+// them, or, in onepass_kernel, again from its start.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

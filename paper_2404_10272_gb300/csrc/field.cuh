@@ -523,11 +523,11 @@ __device__ __forceinline__ void sums_clear(BlobSums& S) {
 // and as a sum: 1.9e-7 and 1.1e-7 on object frames, 6.1e-7 and 2.7e-7 on
 // unbounded ones.  Only the lane's own four samples are a product: with an
 // exponential for each, the compositor was 7 % slower for the same error.
-// A faint ray's opacity is the exception: it is taken as 1 minus a product of
-// (1 - alpha) in a fixed order, that of faint_chunk for stored samples and up
-// to kAllBlobs blobs, else that of faint_product, chunk after chunk.  The roundings above are
-// 2e-4 of so small an opacity, and callers may compare frames with stored ones
-// by their values: so its roundings stay what they were.
+// A faint ray's opacity is the exception: it is 1 minus a product of (1 -
+// alpha) in a fixed order, that of faint_chunk for stored samples and up to
+// kAllBlobs blobs, else that of faint_product, chunk after chunk.  The roundings
+// above are up to 2e-4 of so small an opacity, and another order, or the sum,
+// would move frames that programs have stored by as much; the products keep them.
 constexpr float kFaintDepth = 0.029146346f;  // -log2(0.98)
 constexpr float kNoDepth = 1.f / (1 << 26);  // below it every 1 - alpha of a ray is 1
 
